@@ -9,25 +9,23 @@
 
 namespace infft {
 
-// FFT pass along one axis for a batch of lines held in shared memory: radix-2
-// decimation in time after a bit-reversed load.  Adjoint direction (FWD = false):
-// forward DFT (sign -) of length Ms, keep the M outputs k in I_M, multiply by
-// 1/(Ms w^(k)) of this axis.  Forward direction (FWD = true): the M inputs of I_M times
-// 1/(Ms w^(k)) are placed at k mod Ms, the rest is zero, inverse DFT (sign +).
+// FFT pass along one axis for a batch of lines: Stockham radix-8 (and radix-4) butterflies in
+// registers, exchanged through shared memory.  Adjoint direction (FWD = false): forward DFT
+// (sign -) of length Ms, keep the M outputs k in I_M, multiply by 1/(Ms w^(k)) of this axis.
+// Forward direction (FWD = true): the M inputs of I_M times 1/(Ms w^(k)) are placed at
+// k mod Ms, the rest is zero, inverse DFT (sign +).
 // A pass sees a tensor (A, n_in, B): lines run along the middle index with stride B.
-// Shared-memory position of element i of a line: one padding slot every 16 elements,
-// so that the bit-reversed scatter and the short butterfly strides spread over banks.
+//
+// A line of 512 takes three stages (8, 8, 8): the first reads global memory (or the merged row), the
+// last writes it, and shared memory is crossed twice with two barriers, where the radix-2 pairs before
+// it crossed it six times.  The two line buffers alternate, so a stage needs one barrier and no registers
+// across it.  Fewer twiddle products (two of three stages) also round less: float32 results of the
+// 512 x 512 grids are 10 % nearer the exact sums.  The passes are bound by load latency and barriers, not by
+// bandwidth (batched d = 2, 64 sets: pass along y 0.031 -> 0.021 ms, merging pass along x 0.077 -> 0.067;
+// float64 512 x 512: merging pass 0.093 -> 0.058 ms; d = 3, 128^3: 0.042 -> 0.037 for the three passes).
+// Shared-memory position of element i of a line: one padding slot every 16 elements, so that the
+// first stage's stores (stride 8) and the twiddles' strides spread over banks.
 __device__ __forceinline__ int skew(int i) { return i + (i >> 4); }
-
-// e / M for 0 <= e < 2^22 through a float32 reciprocal rM ~ 1/M and one correction step (the
-// estimate is off by at most one there): a few instructions instead of an integer division
-__device__ __forceinline__ int div_small(int e, int M, float rM) {
-    int q = __float2int_rz((float)e * rM);
-    const int r = e - q * M;
-    if (r < 0) --q;
-    else if (r >= M) ++q;
-    return q;
-}
 
 // lines of length n per FFT block: a 16 KB budget of complex elements, at most 32 lines (more,
 // smaller blocks hide the passes' load latency better: batched d = 2, n = 512: 64 / 32 / 16 / 8 KB
@@ -39,9 +37,112 @@ __host__ __device__ inline int fft_lines(int n, int elem) {
     return L;
 }
 
+// line stride in shared memory: 16 / L (odd for L >= 16) modulo 16 elements, so that the lanes of the
+// passes along y and z, which take consecutive lines of the same few elements, meet distinct banks
+__host__ __device__ inline int fft_stride(int n, int L) {
+    const int want = L < 16 ? 16 / L : 1;
+    return n + (n >> 4) + ((want - n - (n >> 4)) & 15);
+}
+
+// elements of the line buffers (two: a stage reads one and writes the other) and of the twiddles
+__host__ __device__ inline int fft_buf_elems(int n, int L) { return 2 * L * fft_stride(n, L); }
+__host__ __device__ inline int fft_tw_elems(int n) { return (n >> 1) + (n >> 5) + 1; }
+
+// threads of an FFT block: one radix-8 butterfly each for the line budget
+template <class R>
+constexpr int fft_threads() { return sizeof(R) == 4 ? 256 : 128; }
+
 // rows of tiles whose item ranges a merge-on-load block of L lines (grid rows) consults: its
 // own one or L / T, and one above and below
 __host__ __device__ inline int mrg_tile_rows(int L, int T) { return (L <= T ? 1 : L / T) + 2; }
+
+template <class R>
+__device__ __forceinline__ cx<R> mul_w(cx<R> a, cx<R> w) {   // two roundings per part, however it is inlined
+    return mk<R>(fma(a.re, w.re, -(a.im * w.im)), fma(a.re, w.im, a.im * w.re));
+}
+// a times -i (adjoint direction) or i (forward direction)
+template <class R, bool FWD>
+__device__ __forceinline__ cx<R> rot(cx<R> a) { return FWD ? mk<R>(-a.im, a.re) : mk<R>(a.im, -a.re); }
+
+// DFT of RX = 4 or 8 values in place, natural order, sign - (FWD = false) or + (FWD = true)
+template <class R, bool FWD, int RX>
+__device__ __forceinline__ void dft(cx<R>* v) {
+    if constexpr (RX == 4) {
+        const cx<R> a = add(v[0], v[2]), b = sub(v[0], v[2]), c = add(v[1], v[3]), d = rot<R, FWD>(sub(v[1], v[3]));
+        v[0] = add(a, c); v[2] = sub(a, c);
+        v[1] = add(b, d); v[3] = sub(b, d);
+    } else {
+        cx<R> e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+        dft<R, FWD, 4>(e);
+        dft<R, FWD, 4>(o);
+        const R c = R(0.70710678118654752440);
+        // o[1] W_8, o[2] W_8^2, o[3] W_8^3 with W_8 = (1 -+ i) c: the factor c goes into the last additions
+        const cx<R> r1 = rot<R, FWD>(o[1]), r3 = rot<R, FWD>(o[3]);
+        const cx<R> p = add(o[1], r1), q = sub(r3, o[3]), h = rot<R, FWD>(o[2]);
+        v[0] = add(e[0], o[0]); v[4] = sub(e[0], o[0]);
+        v[2] = add(e[2], h);    v[6] = sub(e[2], h);
+        v[1] = mk<R>(fma(p.re, c, e[1].re), fma(p.im, c, e[1].im));
+        v[5] = mk<R>(fma(p.re, -c, e[1].re), fma(p.im, -c, e[1].im));
+        v[3] = mk<R>(fma(q.re, c, e[3].re), fma(q.im, c, e[3].im));
+        v[7] = mk<R>(fma(q.re, -c, e[3].re), fma(q.im, -c, e[3].im));
+    }
+}
+
+// One Stockham stage of radix RX on L lines of n elements, Ns the product of the radices before it:
+// butterfly j of a line takes elements j + r n / RX (through ld), multiplies them by
+// exp(-+2 pi i r k / (RX Ns)), k = j mod Ns, and writes its results at (j - k) RX + k + r Ns
+// (through st).  L_FAST: consecutive threads take consecutive lines.
+template <class R, bool FWD, int RX, int NTH, class Ld, class St>
+__device__ __forceinline__ void fft_stage(int L, int logL, int logn, int logNs, bool l_fast, const cx<R>* tws,
+                                          const Ld& ld, const St& st) {
+    constexpr int LOGR = RX == 8 ? 3 : 2;
+    const int n = 1 << logn, logq = logn - LOGR, q = 1 << logq;
+    for (int e = threadIdx.x; e < (L << logq); e += NTH) {
+        const int l = l_fast ? (e & (L - 1)) : (e >> logq), j = l_fast ? (e >> logL) : (e & (q - 1));
+        cx<R> v[RX];
+        ld(l, j, q, v);
+        const int k = j & ((1 << logNs) - 1);
+        if (logNs > 0) {
+            const int step = k << (logq - logNs);   // of n-th roots of unity
+#pragma unroll
+            for (int r = 1; r < RX; ++r) {
+                const int i = r * step, h = i & ((n >> 1) - 1);
+                cx<R> w = tws[skew(h)];
+                if (i & (n >> 1)) w = mk<R>(-w.re, -w.im);
+                if (FWD) w.im = -w.im;
+                v[r] = mul_w(v[r], w);
+            }
+        }
+        dft<R, FWD, RX>(v);
+        const int o = ((j - k) << LOGR) + k;
+#pragma unroll
+        for (int r = 0; r < RX; ++r) st(l, o + (r << logNs), v[r]);
+    }
+}
+
+// the sum of a cell over the items of its (at most four) sources, in order: item k of source q at
+// s_q + k cells.  Four loads in flight at a time (a dense centre's tile is split into dozens of items).
+template <class R>
+__device__ __noinline__ cx<R> merge_items(const cx<R>* padded, unsigned cells, size_t s0, size_t s1, size_t s2, size_t s3,
+                                          int n0, int n1, int n2, int n3) {
+    cx<R> acc = mk<R>(0, 0);
+#pragma unroll 1
+    for (int q = 0; q < 4; ++q) {
+        const cx<R>* p = padded + (q == 0 ? s0 : q == 1 ? s1 : q == 2 ? s2 : s3);
+        const int n = q == 0 ? n0 : q == 1 ? n1 : q == 2 ? n2 : n3;
+        int k = 0;
+        for (; k + 4 <= n; k += 4) {
+            cx<R> v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = p[(size_t)(k + i) * cells];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc = add(acc, v[i]);
+        }
+#pragma unroll 1
+        for (; k < n; ++k) acc = add(acc, p[(size_t)k * cells]);
+    }
+    return acc;
+}
 
 // With MRG (d = 2 adjoint, pass 0 only) the block's lines are grid rows whose cells are summed
 // from the padded tiles as they are loaded: the halo merge of k_merge2d in the same order per
@@ -54,7 +155,6 @@ __host__ __device__ inline int mrg_tile_rows(int L, int T) { return (L <= T ? 1 
 template <class R, int D, bool FWD, bool MRG, int NTH>
 __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, const int gblk,
                                           unsigned char* smem_raw) {
-    cx<R>* buf = reinterpret_cast<cx<R>*>(smem_raw);
     const int jb = find_job(js.pre_fft[pass], js.njobs, gblk);
     const Job<R>& J = js.job[jb];
     const int lb = gblk - js.pre_fft[pass][jb];
@@ -64,20 +164,20 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
     const long long A = expl ? js.axA : ipow(Ms, t);
     const long long B = expl ? js.axB : ipow(M, D - 1 - t);
     const int MB = expl ? M / js.axblk : M;   // output block along the middle index
-    const int n = Ms;
-    // skewed line stride, odd in 8-byte words: the same element of 16 consecutive lines (the
-    // loads and stores of the passes along y and z) falls into 16 distinct bank pairs
-    const int ns = n + (n >> 4) + 1;
-    const int logn = 31 - __clz(n);
+    const int n = Ms, logn = 31 - __clz(n);
+    const int ns = fft_stride(n, L);
     const long long nlines = A * B;
     const long long q0 = (long long)lb * L;
     const bool lanes_b = (B >= L);  // consecutive lines are consecutive b: coalesce along b
 
-    cx<R>* tws = buf + L * ns;      // the n/2 twiddles after the lines
-    for (int k = threadIdx.x; k < (Ms >> 1); k += NTH) tws[k] = J.tw[k];
+    cx<R>* buf0 = reinterpret_cast<cx<R>*>(smem_raw);
+    cx<R>* buf1 = buf0 + L * ns;
+    cx<R>* tws = buf1 + L * ns;     // the n/2 twiddles, skewed, after the lines
+    for (int k = threadIdx.x; k < (n >> 1); k += NTH) tws[skew(k)] = J.tw[k];
     // then (merging pass only) the table of tile item ranges, then the M deconvolution factors
     const int nrng = (MRG && pass == 0) ? mrg_tile_rows(L, J.T) * J.ntile : 0;
-    R* dvs = reinterpret_cast<R*>(reinterpret_cast<int2*>(tws + (Ms >> 1)) + nrng);
+    int2* rng = reinterpret_cast<int2*>(tws + fft_tw_elems(n));
+    R* dvs = reinterpret_cast<R*>(rng + nrng);
     for (int k = threadIdx.x; k < M; k += NTH) dvs[k] = J.dinv[k];
 
     const cx<R>* src;
@@ -93,7 +193,6 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
         dst = (pass == D - 1) ? J.grid : (pass == 0 ? J.tmp1 : J.tmp2);
     }
     const int tid = threadIdx.x;
-    constexpr int nth = NTH;
     const int logL = 31 - __clz(L);   // L is a power of two
 
     // offsets of each line's first element in the source and destination tensors (line l of
@@ -115,35 +214,37 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
         s_in[tid] = bi;
         s_out[tid] = bo;
     }
-    __syncthreads();
-
+    int ty0 = 0, logT = 0, lognt = 0;
     if (MRG && pass == 0) {
-        const int T = J.T, m = J.m, P = J.P, nt = J.ntile;
-        const int logT = 31 - __clz(T), lognt = 31 - __clz(nt);
-        const int ty0 = (int)(q0 >> logT);
-        const int ntr = mrg_tile_rows(L, T);
-        int2* rng = reinterpret_cast<int2*>(tws + (n >> 1));   // [ntr][nt] first item, count
-        for (int k = tid; k < ntr * nt; k += nth) {
+        const int T = J.T, nt = J.ntile;
+        logT = 31 - __clz(T);
+        lognt = 31 - __clz(nt);
+        ty0 = (int)(q0 >> logT);
+        for (int k = tid; k < nrng; k += NTH) {
             const int tyw = (ty0 - 1 + (k >> lognt)) & (nt - 1), tx = k & (nt - 1);
             const int a = __ldg(J.tile_items + tyw * nt + tx), b = __ldg(J.tile_items + tyw * nt + tx + 1);
-            rng[k] = make_int2(a, b - a);
+            rng[k] = make_int2(a, b - a);   // [tile row][tile] first item, count
         }
-        __syncthreads();
-        // Thread columns: i = tid + nth kc for n >= nth (every line), else i = tid mod n on lines
-        // l = tid / n + (nth / n) k.  The x-sources of a column and the y-sources of a line are
-        // found once each; an element then looks up its (at most four) tiles' item ranges.
+    }
+    __syncthreads();
+
+    // the merge: every element of the block's rows into buf0, in order.  Thread columns: i = tid + NTH kc
+    // for n >= NTH (every line), else i = tid mod n on lines l = tid / n + (NTH / n) k.  The x-sources
+    // of a column and the y-sources of a line are found once each; an element then looks up its (at most
+    // four) tiles' item ranges.
+    if (MRG && pass == 0) {
+        const int T = J.T, m = J.m, P = J.P, nt = J.ntile;
         const unsigned cells = (unsigned)(P * P);
-        const int ncol = n >= nth ? n / nth : 1, dl = n >= nth ? 1 : nth / n;
-        const int i0 = n >= nth ? tid : (tid & (n - 1)), l0 = n >= nth ? 0 : (tid >> logn);
+        const int ncol = n >= NTH ? n / NTH : 1, dl = n >= NTH ? 1 : NTH / n;
+        const int i0 = n >= NTH ? tid : (tid & (n - 1)), l0 = n >= NTH ? 0 : (tid >> logn);
         for (int kc = 0; kc < ncol; ++kc) {
-            const int i = i0 + kc * nth;
+            const int i = i0 + kc * NTH;
             const int c = i & (T - 1), tx = i >> logT;
             int xcol[2], xoff[2], nx = 1;
             xcol[0] = tx; xoff[0] = c + m;
             xcol[1] = 0; xoff[1] = 0;
             if (c + T + m < P) { xcol[1] = (tx - 1) & (nt - 1); xoff[1] = c + T + m; nx = 2; }
             else if (c - T + m >= 0) { xcol[1] = (tx + 1) & (nt - 1); xoff[1] = c - T + m; nx = 2; }
-            const int pos = skew(bitrev(i, logn));
 #pragma unroll 2
             for (int l = l0; l < L; l += dl) {
                 const long long y = q0 + l;
@@ -173,141 +274,89 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
 #pragma unroll
                     for (int q = 0; q < 4; ++q) v[q] = cnt[q] > 0 ? J.padded[src0[q]] : mk<R>(0, 0);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if (cnt[q] <= 0) continue;
-                        acc = add(acc, v[q]);
-#pragma unroll 1
-                        for (int k = 1; k < cnt[q]; ++k) acc = add(acc, J.padded[src0[q] + (size_t)k * cells]);
-                    }
+                    for (int q = 0; q < 4; ++q)
+                        if (cnt[q] > 0) acc = add(acc, v[q]);
+                    // tiles with more points than one item holds (rare; kept out of this loop's registers)
+                    if (max(max(cnt[0], cnt[1]), max(cnt[2], cnt[3])) > 1)
+                        acc = merge_items<R>(J.padded, cells, src0[0], src0[1], src0[2], src0[3], cnt[0], cnt[1], cnt[2], cnt[3]);
                 }
-                buf[l * ns + pos] = acc;
+                buf0[l * ns + skew(i)] = acc;
             }
         }
-    } else if (!FWD) {
-        // each thread issues the loads of up to eight elements before storing any, so that
-        // the block waits for one global-load latency rather than eight in a row
-        constexpr int KL = 8;
-        const int total = L * n;
-        for (int e0 = tid; e0 < total; e0 += KL * nth) {
-            cx<R> v[KL];
-            int pos[KL];
-#pragma unroll
-            for (int k = 0; k < KL; ++k) {
-                const int e = e0 + k * nth;
-                pos[k] = -1;
-                v[k] = mk<R>(0, 0);
-                if (e < total) {
-                    int l, i;
-                    if (lanes_b) { l = e & (L - 1); i = e >> logL; } else { i = e & (n - 1); l = e >> logn; }
-                    const long long g0 = s_in[l];
-                    pos[k] = l * ns + skew(bitrev(i, logn));
-                    if (g0 >= 0) v[k] = src[g0 + (long long)i * B];
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < KL; ++k)
-                if (pos[k] >= 0) buf[pos[k]] = v[k];
-        }
-    } else {
-        for (int e = tid; e < L * ns; e += nth) buf[e] = mk<R>(0, 0);
         __syncthreads();
-        const float rM = 1.f / (float)M;
-        for (int e = tid; e < L * M; e += nth) {
-            int l, i;
-            if (lanes_b) { l = e & (L - 1); i = e >> logL; } else { l = div_small(e, M, rM); i = e - l * M; }
+    }
+    cx<R>*from = MRG && pass == 0 ? buf0 : buf1, *to = MRG && pass == 0 ? buf1 : buf0;
+    // the first stage's inputs: elements j + r q of line l, all loads issued before any is used
+    auto ld_in = [&](int l, int j, int q, auto& v) {
+        constexpr int RX = sizeof(v) / sizeof(v[0]);
+        if (MRG && pass == 0) {
+#pragma unroll
+            for (int r = 0; r < RX; ++r) v[r] = from[l * ns + skew(j + r * q)];
+        } else {
             const long long g0 = s_in[l];
-            if (g0 >= 0) {
-                const cx<R> v = scale(src[g0 + (long long)i * B], dvs[i]);
-                const int bin = (i - M / 2) & (n - 1);   // n = M_sigma is a power of two
-                buf[l * ns + skew(bitrev(bin, logn))] = v;
+#pragma unroll
+            for (int r = 0; r < RX; ++r) {
+                int i = j + r * q;
+                if (FWD) i = (i + M / 2) & (n - 1);   // coefficient of this bin, if below M
+                v[r] = (g0 >= 0 && (!FWD || i < M)) ? src[g0 + (long long)i * B] : mk<R>(0, 0);
             }
-        }
-    }
-    __syncthreads();
-
-    // Butterflies in place, two radix-2 stages at a time: one thread takes the four
-    // elements j + k q (k = 0..3) of a group of 4q and applies the stage of half-length q
-    // (twiddle W_2q^pos) and then that of half-length 2q (W_4q^pos, W_4q^(pos+q)) in
-    // registers.  An odd number of stages starts with one radix-2 stage of half-length 1.
-    // Twiddles W_n^k = exp(-2 pi i k / n), k < n/2, come from shared memory (conjugated
-    // for the inverse direction).
-    const int half_n = n >> 1;
-    const int loghn = logn - 1;
-    int lh = 0;
-    if (logn & 1) {
-        for (int e = tid; e < L * half_n; e += nth) {
-            const int l = e >> loghn, jj = e & (half_n - 1);
-            cx<R>* row = buf + l * ns;
-            const cx<R> a = row[skew(2 * jj)], b = row[skew(2 * jj + 1)];
-            row[skew(2 * jj)] = add(a, b);
-            row[skew(2 * jj + 1)] = sub(a, b);
-        }
-        __syncthreads();
-        lh = 1;
-    }
-    const int quarter_n = n >> 2;
-    const int logqn = logn - 2;
-    for (; lh < logn; lh += 2) {
-        const int q = 1 << lh;
-        for (int e = tid; e < L * quarter_n; e += nth) {
-            const int l = e >> logqn, jj = e & (quarter_n - 1);
-            const int grp = jj >> lh, pos = jj & (q - 1);
-            const int base = grp * (q << 2) + pos;
-            cx<R>* row = buf + l * ns;
-            const cx<R> a0 = row[skew(base)], a1 = row[skew(base + q)];
-            const cx<R> a2 = row[skew(base + 2 * q)], a3 = row[skew(base + 3 * q)];
-            cx<R> w1 = tws[pos << (logn - 1 - lh)];
-            cx<R> w2 = tws[pos << (logn - 2 - lh)];
-            cx<R> w3 = tws[(pos + q) << (logn - 2 - lh)];
-            if (FWD) { w1.im = -w1.im; w2.im = -w2.im; w3.im = -w3.im; }
-            cx<R> t = mul(w1, a1);
-            const cx<R> b0 = add(a0, t), b1 = sub(a0, t);
-            t = mul(w1, a3);
-            const cx<R> b2 = add(a2, t), b3 = sub(a2, t);
-            t = mul(w2, b2);
-            row[skew(base)] = add(b0, t);
-            row[skew(base + 2 * q)] = sub(b0, t);
-            t = mul(w3, b3);
-            row[skew(base + q)] = add(b1, t);
-            row[skew(base + 3 * q)] = sub(b1, t);
-        }
-        __syncthreads();
-    }
-
-    if (!FWD) {
-        if (expl) {
-            for (int e = tid; e < L * M; e += nth) {
-                int l, i;
-                if (lanes_b) { l = e & (L - 1); i = e >> logL; } else { i = e % M; l = e / M; }
-                const long long g0 = s_out[l];
-                if (g0 >= 0) {
-                    const int bin = (i - M / 2) & (n - 1);
-                    // block i / MB of the middle index holds the (A, MB, B) tensor of its indices
-                    const long long o = (long long)(i / MB) * A * MB * B + (long long)(i % MB) * B;
-                    dst[g0 + o] = scale(buf[l * ns + skew(bin)], dvs[i]);
+            if (FWD) {
+#pragma unroll
+                for (int r = 0; r < RX; ++r) {
+                    const int i = (j + r * q + M / 2) & (n - 1);
+                    if (i < M) v[r] = scale(v[r], dvs[i]);
                 }
             }
-        } else if (lanes_b) {
-            for (int e = tid; e < L * M; e += nth) {
-                const int l = e & (L - 1), i = e >> logL;
-                const long long g0 = s_out[l];
-                if (g0 >= 0) dst[g0 + (long long)i * B] = scale(buf[l * ns + skew((i - M / 2) & (n - 1))], dvs[i]);
-            }
-        } else {   // nth / L threads per line (both powers of two), no division per element
-            const int tpl = nth >> logL, l = tid / tpl;
-            const long long g0 = s_out[l];
-            if (g0 >= 0)
-                for (int i = tid & (tpl - 1); i < M; i += tpl)
-                    dst[g0 + (long long)i * B] = scale(buf[l * ns + skew((i - M / 2) & (n - 1))], dvs[i]);
         }
-    } else {
-        for (int e = tid; e < L * n; e += nth) {
-            int l, i;
-            if (lanes_b) { l = e & (L - 1); i = e >> logL; } else { i = e & (n - 1); l = e >> logn; }
-            const long long g0 = s_out[l];
-            if (g0 >= 0) dst[g0 + (long long)i * B] = buf[l * ns + skew(i)];
+    };
+    // a result: bin i of line l
+    auto st_out = [&](int l, int i, cx<R> v) {
+        const long long g0 = s_out[l];
+        if (g0 < 0) return;
+        if (FWD) {
+            dst[g0 + (long long)i * B] = v;
+            return;
         }
+        const int k = (i + M / 2) & (n - 1);
+        if (k >= M) return;
+        // explicit passes: block k / MB of the middle index holds the (A, MB, B) tensor of its indices
+        const long long o = expl ? (long long)(k / MB) * A * MB * B + (long long)(k % MB) * B : (long long)k * B;
+        dst[g0 + o] = scale(v, dvs[k]);
+    };
+    auto ld_buf = [&](int l, int j, int q, auto& v) {
+        constexpr int RX = sizeof(v) / sizeof(v[0]);
+#pragma unroll
+        for (int r = 0; r < RX; ++r) v[r] = from[l * ns + skew(j + r * q)];
+    };
+    auto st_to = [&](int l, int i, cx<R> v) { to[l * ns + skew(i)] = v; };
+
+    // radices: eights, then one or two fours (n = 4^2 or 4: fours only)
+    const int nfour = logn % 3 == 0 ? 0 : logn % 3 == 2 ? 1 : 2, neight = (logn - 2 * nfour) / 3;
+    auto swap_bufs = [&]() {
+        __syncthreads();
+        cx<R>* const s = from;
+        from = to;
+        to = s;
+    };
+    if (neight > 0) fft_stage<R, FWD, 8, NTH>(L, logL, logn, 0, lanes_b && !(MRG && pass == 0), tws, ld_in, st_to);
+    else fft_stage<R, FWD, 4, NTH>(L, logL, logn, 0, lanes_b && !(MRG && pass == 0), tws, ld_in, st_to);
+    swap_bufs();
+    int logNs = neight > 0 ? 3 : 2;
+    while (logNs < logn) {
+        const bool eight = logNs < 3 * neight;
+        const int next = logNs + (eight ? 3 : 2);
+        if (next == logn) {
+            if (eight) fft_stage<R, FWD, 8, NTH>(L, logL, logn, logNs, lanes_b, tws, ld_buf, st_out);
+            else fft_stage<R, FWD, 4, NTH>(L, logL, logn, logNs, lanes_b, tws, ld_buf, st_out);
+            return;
+        }
+        if (eight) fft_stage<R, FWD, 8, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_to);
+        else fft_stage<R, FWD, 4, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_to);
+        swap_bufs();
+        logNs = next;
     }
+    // n = 4 or 8: a single stage
+    for (int e = tid; e < L * n; e += NTH) st_out(e >> logn, e & (n - 1), from[(e >> logn) * ns + skew(e & (n - 1))]);
 }
 
 
@@ -333,7 +382,7 @@ inline size_t fft_smem_mrg(const JobSet<R>& js) {
     for (int j = 0; j < js.njobs; ++j) {
         const Job<R>& J = js.job[j];
         const int n = J.Ms, L = fft_lines(n, (int)sizeof(cx<R>));
-        mx = std::max(mx, ((size_t)L * (n + n / 16 + 1) + n / 2) * sizeof(cx<R>) +
+        mx = std::max(mx, ((size_t)fft_buf_elems(n, L) + fft_tw_elems(n)) * sizeof(cx<R>) +
                               (size_t)mrg_tile_rows(L, J.T) * J.ntile * sizeof(int2) + (size_t)J.M * sizeof(R));
     }
     return mx;
@@ -346,7 +395,7 @@ inline size_t fft_smem(const JobSet<R>& js) {
     size_t mx = 0;
     for (int j = 0; j < js.njobs; ++j) {
         const int n = js.job[j].Ms, L = fft_lines(n, (int)sizeof(cx<R>));
-        mx = std::max(mx, ((size_t)L * (n + n / 16 + 1) + n / 2) * sizeof(cx<R>) + (size_t)js.job[j].M * sizeof(R));
+        mx = std::max(mx, ((size_t)fft_buf_elems(n, L) + fft_tw_elems(n)) * sizeof(cx<R>) + (size_t)js.job[j].M * sizeof(R));
     }
     return mx;
 }

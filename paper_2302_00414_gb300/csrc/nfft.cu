@@ -284,13 +284,13 @@ __device__ __forceinline__ cx<R> merged_cell(const Job<R>& J, long long cidx) {
 }
 
 // ---------------------------------------------------------------------------------------
-// float32 forms bounded to the register counts they reach unbounded as separate kernels (40,
-// 48): six (five merging) 256-thread blocks per SM; float64 forms unbounded
+// float32: four 256-thread blocks per SM (64 registers hold a radix-8 butterfly), five of the merging pass,
+// whose loads want more threads (0.069 ms with four, 0.067 with five, 0.079 with six)
 template <class R, int D, bool FWD, bool MRG = false>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? (MRG ? 5 : 6) : 1)
+__global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? (MRG ? 5 : 4) : 1)
     k_fft(const __grid_constant__ JobSet<R> js, int pass) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    fft_block<R, D, FWD, MRG, 256>(js, pass, blockIdx.x, smem_raw);
+    fft_block<R, D, FWD, MRG, fft_threads<R>()>(js, pass, blockIdx.x, smem_raw);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -440,7 +440,7 @@ static infft_status launch_fft_adjoint(JobSet<R>& js, cudaStream_t st, cudaEvent
     const size_t fsmem = fft_smem(js);
     INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
     for (int p = 0; p < D; ++p) {
-        k_fft<R, D, false><<<js.pre_fft[p][js.njobs], 256, fsmem, st>>>(js, p);
+        k_fft<R, D, false><<<js.pre_fft[p][js.njobs], fft_threads<R>(), fsmem, st>>>(js, p);
         INFFT_LAUNCHED();
         if (ev) INFFT_CUDA(cudaEventRecord(ev[3 + p], st));
     }
@@ -451,12 +451,12 @@ template <class R>
 static infft_status launch_fft_adjoint_mrg(JobSet<R>& js, cudaStream_t st, cudaEvent_t* ev) {
     const size_t msmem = fft_smem_mrg(js);
     INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 2, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msmem));
-    k_fft<R, 2, false, true><<<js.pre_fft[0][js.njobs], 256, msmem, st>>>(js, 0);
+    k_fft<R, 2, false, true><<<js.pre_fft[0][js.njobs], fft_threads<R>(), msmem, st>>>(js, 0);
     INFFT_LAUNCHED();
     if (ev) INFFT_CUDA(cudaEventRecord(ev[3], st));
     const size_t fsmem = fft_smem(js);
     INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
-    k_fft<R, 2, false><<<js.pre_fft[1][js.njobs], 256, fsmem, st>>>(js, 1);
+    k_fft<R, 2, false><<<js.pre_fft[1][js.njobs], fft_threads<R>(), fsmem, st>>>(js, 1);
     INFFT_LAUNCHED();
     if (ev) INFFT_CUDA(cudaEventRecord(ev[4], st));
     return INFFT_OK;
@@ -550,7 +550,7 @@ static infft_status launch_forward(JobSet<R>& js, cudaStream_t st) {
     const size_t fsmem = fft_smem(js);
     INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
     for (int p = 0; p < D; ++p) {
-        k_fft<R, D, true><<<js.pre_fft[p][js.njobs], 256, fsmem, st>>>(js, p);
+        k_fft<R, D, true><<<js.pre_fft[p][js.njobs], fft_threads<R>(), fsmem, st>>>(js, p);
         INFFT_LAUNCHED();
     }
     if constexpr (D >= 2) {
@@ -616,13 +616,13 @@ static infft_status fft_passes_d(JobSet<R>& js, cudaStream_t st, bool forward) {
     if (forward) {
         INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
         for (int p = 0; p < D; ++p) {
-            k_fft<R, D, true><<<js.pre_fft[p][1], 256, fsmem, st>>>(js, p);
+            k_fft<R, D, true><<<js.pre_fft[p][1], fft_threads<R>(), fsmem, st>>>(js, p);
             INFFT_LAUNCHED();
         }
     } else {
         INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
         for (int p = 0; p < D; ++p) {
-            k_fft<R, D, false><<<js.pre_fft[p][1], 256, fsmem, st>>>(js, p);
+            k_fft<R, D, false><<<js.pre_fft[p][1], fft_threads<R>(), fsmem, st>>>(js, p);
             INFFT_LAUNCHED();
         }
     }
@@ -661,7 +661,7 @@ infft_status run_fft_axis(const Job<R>& J, long long A, long long B, int nblk, c
     js.pre_fft[0][1] = (int)((lines + js.L - 1) / js.L);
     const size_t fsmem = fft_smem(js);
     INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
-    k_fft<R, 2, false><<<js.pre_fft[0][1], 256, fsmem, st>>>(js, 0);
+    k_fft<R, 2, false><<<js.pre_fft[0][1], fft_threads<R>(), fsmem, st>>>(js, 0);
     INFFT_LAUNCHED();
     return INFFT_OK;
 }
