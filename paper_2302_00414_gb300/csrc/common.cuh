@@ -100,56 +100,66 @@ __device__ __forceinline__ R tap_weight(int kind, R u, int s, int m, R inv_m, R 
 // phi(u + m - s) = sum_k c[k][s] v^k, v = 2u - 1, u in [0, 1], degree WPOLY_DEG, obtained
 // by Chebyshev interpolation in float64 at plan creation (piecewise-polynomial kernel
 // evaluation in the manner of Barnett, Magland and af Klinteberg, SIAM J. Sci. Comput.
-// 2019).  Degree 10 reaches the float32 rounding level of the window.  Tap 0 keeps the
-// exact membership rule: I0(0) = 1 on a grid node, 0 otherwise.
+// 2019).  Degree 10 reaches the float32 rounding level of the window.  The window is even, so
+// tap 2m + 1 - s has the polynomial of tap s in -v: the table holds s = 1..m, and the even and
+// odd parts of one polynomial give both taps (11 multiply-adds for two taps instead of 20).  Tap 0
+// keeps the exact membership rule: I0(0) = 1 on a grid node, 0 otherwise.
 constexpr int WPOLY_DEG = 10;
+// rows of the table: c[0..WPOLY_DEG], then what rounding took from c[0] (every point of a grid node has v = -1
+// along that axis, so the coefficients' errors there do not average out)
+constexpr int WPOLY_ROWS = WPOLY_DEG + 2;
 
-// row stride of the coefficient table: taps padded to a multiple of 4 (16-byte rows)
-__host__ __device__ constexpr int wpoly_stride(int W) { return (W + 3) & ~3; }
+// row stride of the coefficient table (tap s at s - 1), padded to a multiple of 4 (16-byte rows)
+__host__ __device__ constexpr int wpoly_stride(int m) { return (m + 3) & ~3; }
 
-template <int W>
-__device__ __forceinline__ void poly_taps(const float* __restrict__ c, float u, float* out) {
-    constexpr int WP = wpoly_stride(W);
-    const float v = 2.f * u - 1.f;
+// the 2m + 1 taps of NC coordinates at once, two taps s, s + 1 per packed multiply-add; the table's
+// rows are read with 16-byte loads (c 16-byte aligned, best in shared memory: a constant operand would
+// have to be moved to registers for every use)
+template <int MM, int NC>
+__device__ __forceinline__ void poly_taps(const float* __restrict__ c, const float* u, float (*out)[2 * MM + 1]) {
+    constexpr int WP = wpoly_stride(MM);
+    constexpr int NP = WP / 2;   // pairs of taps, padded
+    float2 ev[NC][NP], od[NC][NP];
+    float v[NC];
 #pragma unroll
-    for (int s = 1; s < W; ++s) out[s] = c[WPOLY_DEG * WP + s];
+    for (int a = 0; a < NC; ++a) v[a] = 2.f * u[a] - 1.f;
 #pragma unroll
-    for (int k = WPOLY_DEG - 1; k >= 0; --k) {
+    for (int k = WPOLY_DEG; k >= 0; --k) {
 #pragma unroll
-        for (int s = 1; s < W; ++s) out[s] = fmaf(out[s], v, c[k * WP + s]);
-    }
-    out[0] = (u == 0.f) ? 1.f : 0.f;
-}
-
-// the taps of two coordinates at once, each coefficient row read with 16-byte loads
-// (c must be 16-byte aligned)
-template <int W>
-__device__ __forceinline__ void poly_taps2(const float* __restrict__ c, float u0, float u1, float* o0, float* o1) {
-    constexpr int WP = wpoly_stride(W);
-    // Horner on both coordinates at once: one packed two-wide FMA per tap and degree
-    const float2 vv = make_float2(2.f * u0 - 1.f, 2.f * u1 - 1.f);
-    float2 a[WP];
+        for (int q = 0; q < NP; q += 2) {
+            const int row = k == 0 ? WPOLY_DEG + 1 : k;   // c[0] is added last, its low part first
+            const float4 t = *reinterpret_cast<const float4*>(c + row * WP + 2 * q);
+            const float2 t0 = make_float2(t.x, t.y), t1 = make_float2(t.z, t.w);
 #pragma unroll
-    for (int q = 0; q < WP / 4; ++q) {
-        const float4 t = reinterpret_cast<const float4*>(c + WPOLY_DEG * WP)[q];
-        a[4 * q] = make_float2(t.x, t.x); a[4 * q + 1] = make_float2(t.y, t.y);
-        a[4 * q + 2] = make_float2(t.z, t.z); a[4 * q + 3] = make_float2(t.w, t.w);
-    }
-#pragma unroll
-    for (int k = WPOLY_DEG - 1; k >= 0; --k) {
-#pragma unroll
-        for (int q = 0; q < WP / 4; ++q) {
-            const float4 t = reinterpret_cast<const float4*>(c + k * WP)[q];
-            if (4 * q < W) a[4 * q] = __ffma2_rn(a[4 * q], vv, make_float2(t.x, t.x));
-            if (4 * q + 1 < W) a[4 * q + 1] = __ffma2_rn(a[4 * q + 1], vv, make_float2(t.y, t.y));
-            if (4 * q + 2 < W) a[4 * q + 2] = __ffma2_rn(a[4 * q + 2], vv, make_float2(t.z, t.z));
-            if (4 * q + 3 < W) a[4 * q + 3] = __ffma2_rn(a[4 * q + 3], vv, make_float2(t.w, t.w));
+            for (int a = 0; a < NC; ++a) {
+                float2* p = (k & 1) ? od[a] : ev[a];
+                const float2 ww = make_float2(v[a] * v[a], v[a] * v[a]);
+                p[q] = k >= WPOLY_DEG - 1 ? t0 : __ffma2_rn(p[q], ww, t0);
+                if (2 * q + 2 < MM) p[q + 1] = k >= WPOLY_DEG - 1 ? t1 : __ffma2_rn(p[q + 1], ww, t1);
+            }
         }
     }
 #pragma unroll
-    for (int s = 1; s < W; ++s) { o0[s] = a[s].x; o1[s] = a[s].y; }
-    o0[0] = (u0 == 0.f) ? 1.f : 0.f;
-    o1[0] = (u1 == 0.f) ? 1.f : 0.f;
+    for (int q = 0; 2 * q < MM; ++q) {
+        const float2 t0 = *reinterpret_cast<const float2*>(c + 2 * q);
+#pragma unroll
+        for (int a = 0; a < NC; ++a) ev[a][q] = __fadd2_rn(ev[a][q], t0);
+    }
+#pragma unroll
+    for (int a = 0; a < NC; ++a) {
+#pragma unroll
+        for (int q = 0; 2 * q < MM; ++q) {
+            const float2 x = __ffma2_rn(od[a][q], make_float2(v[a], v[a]), ev[a][q]);
+            const float2 y = __ffma2_rn(od[a][q], make_float2(-v[a], -v[a]), ev[a][q]);
+            out[a][2 * q + 1] = x.x;
+            out[a][2 * MM - 2 * q] = y.x;
+            if (2 * q + 2 <= MM) {
+                out[a][2 * q + 2] = x.y;
+                out[a][2 * MM - 2 * q - 1] = y.y;
+            }
+        }
+        out[a][0] = (u[a] == 0.f) ? 1.f : 0.f;
+    }
 }
 
 // ----------------------------------------------------------------------------------------
@@ -163,6 +173,7 @@ struct Job {
     int nitems, window;        // work items (tile, start, count); window kind
     int mode;                  // INFFT_MODE_*
     int S;                     // B_opt slots per axis (2m+2)
+    int wexp;                  // the window is below 2^wexp
     int prefetch, fused_fft;   // the plan's tuning of these choices (0 = library default)
     R beta, inv_m;
     const int* perm;           // sorted position -> caller's index
@@ -172,10 +183,10 @@ struct Job {
     const cx<R>* coef;         // B_opt coefficients, sorted order, N*S^d (BOPT)
     const int4* items;         // (tile, start, count, 0)
     const int* tile_items;     // ntile^d + 1 prefix of items per tile
-    const R* dinv;             // M entries 1/(Ms w^(k)) (per axis)
-    const float* wpoly;        // (WPOLY_DEG + 1) x (2m+1) window polynomial (float32 KB plans) or null
+    const R* dinv;             // M entries 1/(Ms w^(k)) (per axis); float32: then their low parts
+    const float* wpoly;        // WPOLY_ROWS x wpoly_stride(m) window polynomial (float32 KB plans) or null
     const float* wpoly_h;      // host copy of the same table (read by the launchers only) or null
-    const cx<R>* tw;           // Ms/2 twiddles exp(-2 pi i k / Ms)
+    const cx<R>* tw;           // Ms/2 twiddles exp(-2 pi i k / Ms); float32: then their low parts
     cx<R>* padded;             // nitems * P^d
     cx<R>* grid;               // Ms^d
     cx<R>* tmp1;               // FFT intermediates

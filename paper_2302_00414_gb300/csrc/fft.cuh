@@ -20,7 +20,7 @@ namespace infft {
 // last writes it, and shared memory is crossed twice with two barriers, where the radix-2 pairs before
 // it crossed it six times.  The two line buffers alternate, so a stage needs one barrier and no registers
 // across it.  Fewer twiddle products (two of three stages) also round less: float32 results of the
-// 512 x 512 grids are 10 % nearer the exact sums.  The passes are bound by load latency and barriers, not by
+// 512 x 512 grids are nearer the exact sums.  The passes are bound by load latency and barriers, not by
 // bandwidth (batched d = 2, 64 sets: pass along y 0.031 -> 0.021 ms, merging pass along x 0.077 -> 0.067;
 // float64 512 x 512: merging pass 0.093 -> 0.058 ms; d = 3, 128^3: 0.042 -> 0.037 for the three passes).
 // Shared-memory position of element i of a line: one padding slot every 16 elements, so that the
@@ -46,7 +46,12 @@ __host__ __device__ inline int fft_stride(int n, int L) {
 
 // elements of the line buffers (two: a stage reads one and writes the other) and of the twiddles
 __host__ __device__ inline int fft_buf_elems(int n, int L) { return 2 * L * fft_stride(n, L); }
-__host__ __device__ inline int fft_tw_elems(int n) { return (n >> 1) + (n >> 5) + 1; }
+template <class R>
+__host__ __device__ inline int fft_tw_elems(int n) { return (sizeof(R) == 4 ? 2 : 1) * ((n >> 1) + (n >> 5) + 1); }
+
+// bytes of a deconvolution factor in shared memory (float32 with its low part)
+template <class R>
+constexpr size_t fft_dv_bytes() { return 8; }
 
 // threads of an FFT block: one radix-8 butterfly each for the line budget
 template <class R>
@@ -56,9 +61,26 @@ constexpr int fft_threads() { return sizeof(R) == 4 ? 256 : 128; }
 // own one or L / T, and one above and below
 __host__ __device__ inline int mrg_tile_rows(int L, int T) { return (L <= T ? 1 : L / T) + 2; }
 
+// a w: float64 with two roundings per part; float32 with w = w + wl to twice the precision and the
+// products' errors carried along, so that one rounding is left (the passes wait for loads and barriers,
+// the extra multiply-adds are free, and the twiddles were a third of the passes' float32 error)
 template <class R>
-__device__ __forceinline__ cx<R> mul_w(cx<R> a, cx<R> w) {   // two roundings per part, however it is inlined
-    return mk<R>(fma(a.re, w.re, -(a.im * w.im)), fma(a.re, w.im, a.im * w.re));
+__device__ __forceinline__ cx<R> mul_w(cx<R> a, cx<R> w, cx<R> wl) {
+    if constexpr (sizeof(R) == 8) {
+        return mk<R>(fma(a.re, w.re, -(a.im * w.im)), fma(a.re, w.im, a.im * w.re));
+    } else {
+        const R p = __fmul_rn(a.im, w.im), q = __fmul_rn(a.im, w.re);
+        const R ep = fmaf(a.im, w.im, -p), eq = fmaf(a.im, w.re, -q);
+        const R lr = fmaf(a.re, wl.re, fmaf(-a.im, wl.im, -ep)), li = fmaf(a.re, wl.im, fmaf(a.im, wl.re, eq));
+        const R r = fmaf(a.re, w.re, -p), i = fmaf(a.re, w.im, q);
+        return mk<R>(__fadd_rn(r, lr), __fadd_rn(i, li));
+    }
+}
+// v d, in float32 with d's low part
+template <class R>
+__device__ __forceinline__ cx<R> mul_d(cx<R> v, R d, R dl) {
+    if constexpr (sizeof(R) == 8) return scale(v, d);
+    else return mk<R>(fmaf(v.re, d, __fmul_rn(v.re, dl)), fmaf(v.im, d, __fmul_rn(v.im, dl)));
 }
 // a times -i (adjoint direction) or i (forward direction)
 template <class R, bool FWD>
@@ -97,6 +119,7 @@ __device__ __forceinline__ void fft_stage(int L, int logL, int logn, int logNs, 
                                           const Ld& ld, const St& st) {
     constexpr int LOGR = RX == 8 ? 3 : 2;
     const int n = 1 << logn, logq = logn - LOGR, q = 1 << logq;
+    const int twl = skew(n >> 1) + 1;   // the twiddles' low parts (float32)
     for (int e = threadIdx.x; e < (L << logq); e += NTH) {
         const int l = l_fast ? (e & (L - 1)) : (e >> logq), j = l_fast ? (e >> logL) : (e & (q - 1));
         cx<R> v[RX];
@@ -107,10 +130,10 @@ __device__ __forceinline__ void fft_stage(int L, int logL, int logn, int logNs, 
 #pragma unroll
             for (int r = 1; r < RX; ++r) {
                 const int i = r * step, h = i & ((n >> 1) - 1);
-                cx<R> w = tws[skew(h)];
-                if (i & (n >> 1)) w = mk<R>(-w.re, -w.im);
-                if (FWD) w.im = -w.im;
-                v[r] = mul_w(v[r], w);
+                cx<R> w = tws[skew(h)], wl = sizeof(R) == 4 ? tws[twl + skew(h)] : mk<R>(0, 0);
+                if (FWD) { w.im = -w.im; wl.im = -wl.im; }
+                const cx<R> x = mul_w(v[r], w, wl);
+                v[r] = (i & (n >> 1)) ? mk<R>(-x.re, -x.im) : x;
             }
         }
         dft<R, FWD, RX>(v);
@@ -173,12 +196,15 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
     cx<R>* buf0 = reinterpret_cast<cx<R>*>(smem_raw);
     cx<R>* buf1 = buf0 + L * ns;
     cx<R>* tws = buf1 + L * ns;     // the n/2 twiddles, skewed, after the lines
-    for (int k = threadIdx.x; k < (n >> 1); k += NTH) tws[skew(k)] = J.tw[k];
+    for (int k = threadIdx.x; k < (n >> 1); k += NTH) {
+        tws[skew(k)] = J.tw[k];
+        if (sizeof(R) == 4) tws[skew(n >> 1) + 1 + skew(k)] = J.tw[(n >> 1) + k];
+    }
     // then (merging pass only) the table of tile item ranges, then the M deconvolution factors
     const int nrng = (MRG && pass == 0) ? mrg_tile_rows(L, J.T) * J.ntile : 0;
-    int2* rng = reinterpret_cast<int2*>(tws + fft_tw_elems(n));
+    int2* rng = reinterpret_cast<int2*>(tws + fft_tw_elems<R>(n));
     R* dvs = reinterpret_cast<R*>(rng + nrng);
-    for (int k = threadIdx.x; k < M; k += NTH) dvs[k] = J.dinv[k];
+    for (int k = threadIdx.x; k < (sizeof(R) == 4 ? 2 : 1) * M; k += NTH) dvs[k] = J.dinv[k];
 
     const cx<R>* src;
     cx<R>* dst;
@@ -304,7 +330,7 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
 #pragma unroll
                 for (int r = 0; r < RX; ++r) {
                     const int i = (j + r * q + M / 2) & (n - 1);
-                    if (i < M) v[r] = scale(v[r], dvs[i]);
+                    if (i < M) v[r] = mul_d(v[r], dvs[i], sizeof(R) == 4 ? dvs[M + i] : R(0));
                 }
             }
         }
@@ -321,7 +347,7 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
         if (k >= M) return;
         // explicit passes: block k / MB of the middle index holds the (A, MB, B) tensor of its indices
         const long long o = expl ? (long long)(k / MB) * A * MB * B + (long long)(k % MB) * B : (long long)k * B;
-        dst[g0 + o] = scale(v, dvs[k]);
+        dst[g0 + o] = mul_d(v, dvs[k], sizeof(R) == 4 ? dvs[M + k] : R(0));
     };
     auto ld_buf = [&](int l, int j, int q, auto& v) {
         constexpr int RX = sizeof(v) / sizeof(v[0]);
@@ -382,8 +408,8 @@ inline size_t fft_smem_mrg(const JobSet<R>& js) {
     for (int j = 0; j < js.njobs; ++j) {
         const Job<R>& J = js.job[j];
         const int n = J.Ms, L = fft_lines(n, (int)sizeof(cx<R>));
-        mx = std::max(mx, ((size_t)fft_buf_elems(n, L) + fft_tw_elems(n)) * sizeof(cx<R>) +
-                              (size_t)mrg_tile_rows(L, J.T) * J.ntile * sizeof(int2) + (size_t)J.M * sizeof(R));
+        mx = std::max(mx, ((size_t)fft_buf_elems(n, L) + fft_tw_elems<R>(n)) * sizeof(cx<R>) +
+                              (size_t)mrg_tile_rows(L, J.T) * J.ntile * sizeof(int2) + (size_t)J.M * fft_dv_bytes<R>());
     }
     return mx;
 }
@@ -395,7 +421,7 @@ inline size_t fft_smem(const JobSet<R>& js) {
     size_t mx = 0;
     for (int j = 0; j < js.njobs; ++j) {
         const int n = js.job[j].Ms, L = fft_lines(n, (int)sizeof(cx<R>));
-        mx = std::max(mx, ((size_t)fft_buf_elems(n, L) + fft_tw_elems(n)) * sizeof(cx<R>) + (size_t)js.job[j].M * sizeof(R));
+        mx = std::max(mx, ((size_t)fft_buf_elems(n, L) + fft_tw_elems<R>(n)) * sizeof(cx<R>) + (size_t)js.job[j].M * fft_dv_bytes<R>());
     }
     return mx;
 }

@@ -22,6 +22,7 @@ struct infft_plan_s {
     infft_tune_t tune = {0, 0, 0, 0, 0};   // caller's tuning (0 = library default)
     int logMs;
     double beta;
+    int wexp = 0;             // the window's values are below 2^wexp
 
     // sorted points (device)
     int* perm = nullptr;

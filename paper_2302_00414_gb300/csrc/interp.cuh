@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(128) k_interp_t(const __grid_constant__ JobSet
     float* poly = reinterpret_cast<float*>(pad + ((cells + 1) & ~1));
     const bool use_poly = F32 && J.wpoly != nullptr;
     if (use_poly) {
-        for (int e = lane; e < (WPOLY_DEG + 1) * wpoly_stride(W); e += 32) poly[e] = J.wpoly[e];
+        for (int e = lane; e < WPOLY_ROWS * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
     }
     int tz = 0, ty, tx;
     if (D == 3) { tz = item.x / (nt * nt); ty = (item.x / nt) % nt; tx = item.x % nt; }
@@ -56,25 +56,24 @@ __global__ void __launch_bounds__(128) k_interp_t(const __grid_constant__ JobSet
         const int ox = (int)(cl & (uint32_t)Mmask) - tx * T;
         const int oy = (int)((cl >> logMs) & (uint32_t)Mmask) - ty * T;
         const int oz = D == 3 ? (int)(cl >> (2 * logMs)) - tz * T : 0;
-        R wz[W], wy[W], wx[W];
-        const R uy = J.u[(size_t)i * D + D - 2], ux = J.u[(size_t)i * D + D - 1];
-        const R uz = D == 3 ? J.u[(size_t)i * D] : R(0);
+        R wt[D][W];   // (z,) y, x
+        R uu[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) uu[a] = J.u[(size_t)i * D + a];
         bool done = false;
         if constexpr (F32) {
             if (use_poly) {
-                poly_taps2<W>(poly, uy, ux, wy, wx);
-                if (D == 3) poly_taps<W>(poly, uz, wz);
+                poly_taps<MM, D>(poly, uu, wt);
                 done = true;
             }
         }
         if (!done) {
 #pragma unroll
-            for (int s = 0; s < W; ++s) {
-                wy[s] = tap_weight<R>(J.window, uy, s, MM, J.inv_m, J.beta);
-                wx[s] = tap_weight<R>(J.window, ux, s, MM, J.inv_m, J.beta);
-                if (D == 3) wz[s] = tap_weight<R>(J.window, uz, s, MM, J.inv_m, J.beta);
-            }
+            for (int s = 0; s < W; ++s)
+#pragma unroll
+                for (int a = 0; a < D; ++a) wt[a][s] = tap_weight<R>(J.window, uu[a], s, MM, J.inv_m, J.beta);
         }
+        const R *wz = wt[0], *wy = wt[D - 2], *wx = wt[D - 1];
         cx<R> acc = mk<R>(0, 0);
         const int NZ = D == 3 ? W : 1;
 #pragma unroll 1
@@ -107,7 +106,7 @@ static infft_status launch_interp_t(JobSet<R>& js, cudaStream_t st) {
     int P = 0;
     for (int j = 0; j < js.njobs; ++j) P = std::max(P, js.job[j].P);
     const size_t cells = D == 3 ? (size_t)P * P * P : (size_t)P * P;
-    size_t spw = ((cells + 1) & ~(size_t)1) * sizeof(cx<R>) + (WPOLY_DEG + 1) * wpoly_stride(2 * MM + 1) * sizeof(float);
+    size_t spw = ((cells + 1) & ~(size_t)1) * sizeof(cx<R>) + WPOLY_ROWS * wpoly_stride(MM) * sizeof(float);
     spw = (spw + 15) & ~(size_t)15;
     const size_t smem_cap = 200 * 1024;
     if (spw > smem_cap) {

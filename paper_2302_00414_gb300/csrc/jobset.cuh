@@ -25,10 +25,10 @@ struct JobSet {
     int pre_items[MAXJ + 1];    // prefix of work items
     int pre_merge[MAXJ + 1];    // prefix of merge blocks
     int pre_fft[3][MAXJ + 1];   // prefix of FFT blocks per pass
-    // the float32 window polynomial of every job, when all jobs share one (wtab_ok): read by
-    // the unrolled tap evaluation straight from the parameter block, no shared-memory loads
+    // the float32 window polynomial of every job, when all jobs share one (wtab_ok): the unrolled
+    // tap evaluation takes its coefficients straight from the parameter block as operands
     int wtab_ok;
-    alignas(16) float wtab[(WPOLY_DEG + 1) * 12];
+    alignas(16) float wtab[WPOLY_ROWS * wpoly_stride(8)];
     Job<R> job[MAXJ];
 };
 

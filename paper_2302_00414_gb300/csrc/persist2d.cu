@@ -90,7 +90,7 @@ __global__ void k_persist_reset(const __grid_constant__ JobSet<float> js) {
 }
 
 template <int MM>
-__global__ void __launch_bounds__(PERSIST_THREADS, 5)
+__global__ void __launch_bounds__(PERSIST_THREADS, 3)
     k_adjoint2d_persistent(const __grid_constant__ JobSet<float> js, const __grid_constant__ PersistQueue pq) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_unit;
@@ -112,8 +112,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 5)
             const Job<float>& J = js.job[j];
             const int li = 4 * (su - pq.su_pre[j]) + warp;
             if (li < J.nitems) {
-                spread2d_item<float, MM, false, true>(js, js.pre_items[j] + li,
-                                                      smem_raw + (size_t)warp * js.smem_per_warp);
+                spread2d_mma_item<MM>(js, js.pre_items[j] + li, smem_raw + (size_t)warp * js.smem_per_warp);
                 __threadfence();
                 __syncwarp();
                 if (lane == 0) atomicAdd(job_counters(J), 1);
@@ -191,7 +190,7 @@ static void build_queue(const JobSet<float>& js, int lag, PersistQueue& pq) {
 
 template <int MM>
 static infft_status launch_persist2d(JobSet<float>& js, cudaStream_t st) {
-    spread2d_setup<float, MM, false, true>(js);
+    spread2d_setup<float, MM, false, false>(js);
     const size_t smem = std::max({(size_t)4 * js.smem_per_warp, fft_smem_mrg(js), fft_smem(js)});
     auto kern = k_adjoint2d_persistent<MM>;
     INFFT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -223,8 +222,10 @@ infft_status persist2d_try(JobSet<float>& js, cudaStream_t st, bool* used) {
     if (env_form("INFFT_PERSISTENT") != 1 || js.njobs < 1 || js.axA > 0) return INFFT_OK;
     int m = 0;
     bool bopt = false;
-    if (!spread2d_eligible(js, &m, &bopt) || bopt || !spread2d_pair_m<float>(m)) return INFFT_OK;
-    if (!spread2d_prefetch(js, m) || !merge_on_load_ok(js)) return INFFT_OK;
+    if (!spread2d_eligible(js, &m, &bopt) || bopt || m > 4) return INFFT_OK;
+    if (!merge_on_load_ok(js)) return INFFT_OK;
+    // prefetch = 2 asks for the staged kernels
+    if (js.job[0].prefetch == 2 || (js.job[0].prefetch == 0 && env_form("INFFT_SPREAD2D_PREFETCH") == 0)) return INFFT_OK;
     for (int j = 0; j < js.njobs; ++j) {
         const Job<float>& J = js.job[j];
         if (J.fused_fft == 1 || (J.fused_fft == 0 && env_form("INFFT_FUSED_MERGE_FFT") == 1)) return INFFT_OK;

@@ -263,10 +263,11 @@ __global__ void k_gather(const int* __restrict__ order, int N, int d, const uint
     }
 }
 
-// 1/(M_sigma w^(k)) for k in I_M (one axis of eq. matrix_D) and FFT twiddles exp(-2 pi i k/Ms).
+// 1/(M_sigma w^(k)) for k in I_M (one axis of eq. matrix_D) and FFT twiddles exp(-2 pi i k/Ms); in
+// float32 each table is followed by what rounding took from its entries.
 template <class R>
 __global__ void k_tables(int M, int Ms, int m, int window, double beta, R* __restrict__ dinv,
-                         cx<R>* __restrict__ tw, double* __restrict__ dinv64) {
+                         cx<R>* __restrict__ tw) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < M) {
         const double k = (double)(i - M / 2);
@@ -288,26 +289,26 @@ __global__ void k_tables(int M, int Ms, int m, int window, double beta, R* __res
         }
         const double v = 1.0 / (Ms * wh);
         dinv[i] = (R)v;
-        if (dinv64) dinv64[i] = v;
+        if (sizeof(R) == 4) dinv[M + i] = (R)(v - (double)(R)v);
     }
     if (i < Ms / 2) {
         double s, c;
         sincospi(2.0 * i / Ms, &s, &c);
         tw[i] = mk<R>((R)c, (R)(-s));
+        if (sizeof(R) == 4) tw[Ms / 2 + i] = mk<R>((R)(c - (double)(R)c), (R)((double)(R)s - s));
     }
 }
 
-// Window polynomials for float32 Kaiser-Bessel plans: one thread per tap s = 1..2m
+// Window polynomials for float32 Kaiser-Bessel plans: one thread per tap s = 1..m
 // interpolates phi(u + m - s), u in [0,1], at the WPOLY_DEG+1 Chebyshev points of
 // v = 2u - 1 and rewrites the Chebyshev series in powers of v (float64 throughout).
 __global__ void k_wpoly(int m, double beta, float* __restrict__ coef) {
     constexpr int P1 = WPOLY_DEG + 1;
-    const int W = 2 * m + 1;
-    const int WP = wpoly_stride(W);
-    const int s = threadIdx.x;
-    if (s >= WP) return;
-    if (s == 0 || s >= W) {  // tap 0 keeps the exact rule; padding slots are zero
-        for (int k = 0; k < P1; ++k) coef[k * WP + s] = 0.f;
+    const int WP = wpoly_stride(m);
+    const int i = threadIdx.x, s = i + 1;
+    if (i >= WP) return;
+    if (s > m) {  // padding slots are zero
+        for (int k = 0; k < WPOLY_ROWS; ++k) coef[k * WP + i] = 0.f;
         return;
     }
     double fv[P1], c[P1], a[P1], tp[P1], tc[P1], tn[P1];
@@ -331,7 +332,8 @@ __global__ void k_wpoly(int m, double beta, float* __restrict__ coef) {
         for (int k = 0; k < P1; ++k) tn[k] = -tp[k] + ((k > 0) ? 2.0 * tc[k - 1] : 0.0);
         for (int k = 0; k < P1; ++k) { a[k] += c[j] * tn[k]; tp[k] = tc[k]; tc[k] = tn[k]; }
     }
-    for (int k = 0; k < P1; ++k) coef[k * WP + s] = (float)a[k];
+    for (int k = 0; k < P1; ++k) coef[k * WP + i] = (float)a[k];
+    coef[P1 * WP + i] = (float)(a[0] - (double)(float)a[0]);
 }
 
 // ----------------------------------------------------------------------------------------
@@ -346,6 +348,7 @@ Job<R> make_job(const infft_plan_s* p, int mode, const void* in, void* out, int 
     J.P = (mode == INFFT_MODE_BOPT) ? p->P : p->T + 2 * p->m;
     J.nitems = p->nitems; J.window = p->window; J.mode = mode; J.S = p->S;
     J.prefetch = p->tune.prefetch; J.fused_fft = p->tune.fused_fft;
+    J.wexp = p->wexp;
     J.beta = (R)p->beta; J.inv_m = (R)(1.0 / p->m);
     J.perm = p->perm; J.cell = p->cell; J.u = (const R*)p->u;
     J.w = (const cx<R>*)p->w_sorted; J.coef = (const cx<R>*)p->coef;
@@ -499,23 +502,23 @@ static infft_status build_plan(infft_plan_s* p, const double* x_in, cudaStream_t
 
 
     // tables
-    INFFT_TRY(dev_alloc(p, &p->dinv, (size_t)p->M * R_sz));
-    INFFT_TRY(dev_alloc(p, &p->tw, (size_t)(Ms / 2) * C_sz));
+    INFFT_TRY(dev_alloc(p, &p->dinv, (size_t)p->M * (p->fp64 ? 1 : 2) * R_sz));
+    INFFT_TRY(dev_alloc(p, &p->tw, (size_t)(Ms / 2) * (p->fp64 ? 1 : 2) * C_sz));
     const int nt = std::max(p->M, Ms / 2);
     if (p->fp64)
         k_tables<double><<<(nt + 255) / 256, 256, 0, st>>>(p->M, Ms, m, p->window, p->beta, (double*)p->dinv,
-                                                          (cx<double>*)p->tw, nullptr);
+                                                          (cx<double>*)p->tw);
     else
         k_tables<float><<<(nt + 255) / 256, 256, 0, st>>>(p->M, Ms, m, p->window, p->beta, (float*)p->dinv,
-                                                         (cx<float>*)p->tw, nullptr);
+                                                         (cx<float>*)p->tw);
     INFFT_LAUNCHED();
 
     // window polynomials (float32 Kaiser-Bessel plans)
     if (!p->fp64 && p->window == WK_KB && 2 * m + 1 <= 32) {
-        INFFT_TRY(dev_alloc(p, (void**)&p->wpoly, (size_t)(WPOLY_DEG + 1) * wpoly_stride(2 * m + 1) * sizeof(float)));
+        INFFT_TRY(dev_alloc(p, (void**)&p->wpoly, (size_t)WPOLY_ROWS * wpoly_stride(m) * sizeof(float)));
         k_wpoly<<<1, 32, 0, st>>>(m, p->beta, p->wpoly);
         INFFT_LAUNCHED();
-        p->wpoly_host.resize((size_t)(WPOLY_DEG + 1) * wpoly_stride(2 * m + 1));
+        p->wpoly_host.resize((size_t)WPOLY_ROWS * wpoly_stride(m));
         INFFT_CUDA(cudaMemcpyAsync(p->wpoly_host.data(), p->wpoly, p->wpoly_host.size() * sizeof(float),
                                    cudaMemcpyDeviceToHost, st));
     }
@@ -565,6 +568,14 @@ infft_status plan_create(int d, int M, int64_t N, const double* x, double sigma,
     p->d = d; p->M = M; p->Ms = Ms; p->m = m; p->N = N; p->sigma = sigma; p->flags = flags; p->fp64 = fp64;
     p->window = (flags & INFFT_WIN_BSPLINE) ? WK_BSPLINE : ((flags & INFFT_WIN_DIRICHLET) ? WK_DIRICHLET : WK_KB);
     p->beta = M_PI * m * (2.0 - (double)M / Ms);
+    if (p->window == WK_KB) {   // its largest value, I0(beta), by the power series
+        double sum = 1.0, term = 1.0;
+        for (int k = 1; term > 1e-3 * sum || k < 0.5 * p->beta; ++k) {
+            term *= 0.25 * p->beta * p->beta / ((double)k * k);
+            sum += term;
+        }
+        std::frexp(1.01 * sum, &p->wexp);
+    }
     int l = 0;
     while ((1 << l) < Ms) ++l;
     p->logMs = l;

@@ -8,28 +8,17 @@
 #include <type_traits>
 
 #include "spread.cuh"
+#include "spreadmma.cuh"
 
 namespace infft {
 
-// Float32 window modes with m <= 4 spread two points at a time, one per half-warp: lane l
-// owns columns 2 (l mod 16) and 2 (l mod 16) + 1 for the points of its half, and the two
-// halves' partial sums of a cell are added when its row is stored.  A 16-byte load of
-// broadcast coefficients costs two shared-memory wavefronts either way, so each then
-// serves two points; shared-memory wavefronts bound this kernel.
-template <class R, int MM, bool BOPT>
-__host__ __device__ constexpr bool spread2d_pair() { return sizeof(R) == 4 && !BOPT && MM <= 4; }
-template <class R>
-constexpr bool spread2d_pair_m(int m) { return sizeof(R) == 4 && m <= 4; }   // window modes
-// row pitch of the staged psi_x: odd (33) when each lane reads one column, even (34) for
-// the 8-byte column pairs of the paired form
-template <class R, int MM, bool BOPT>
-__host__ __device__ constexpr int spread2d_pitch() { return spread2d_pair<R, MM, BOPT>() ? 34 : 33; }
+// Float32 window modes take the tensor-core form of spreadmma.cuh; the register-row form below serves
+// float64 and the B_opt modes.
+template <class R, bool BOPT>
+__host__ __device__ constexpr bool spread2d_mma() { return sizeof(R) == 4 && !BOPT; }
 
-// row stride (complex elements) of the staged c_j psi_y: W in the paired form, whose rows are
-// read with 8-byte broadcasts (an odd stride of 8-byte words: the staging stores of 32 lanes
-// hit distinct banks), W + 1 elsewhere, whose rows are read with 16-byte broadcasts
-template <class R, int MM, bool BOPT>
-__host__ __device__ constexpr int spread2d_we() { return spread2d_pair<R, MM, BOPT>() ? 2 * MM + 1 : 2 * MM + 2; }
+// row pitch of the staged psi_x (odd: each lane reads one column)
+constexpr int SPREAD2D_PX = 33;
 
 // bytes of the per-warp prefetch slots (w, u pairs, perm, cell of 32 points); a multiple of 16
 template <class R, bool PF>
@@ -40,7 +29,7 @@ __host__ __device__ constexpr size_t spread2d_slot_bytes() {
 // ---------------------------------------------------------------------------------------
 // Two-dimensional spreading with the accumulators in registers.  One warp per work
 // item; lane l owns column l of the item's P x P padded tile (P = T + 2m, one more for
-// B_opt slots; P <= 32), or a column pair in the paired form above.
+// B_opt slots; P <= 32).
 // The item's points are sorted by base row, so the rows a point can touch,
 // [oy, oy + 2m] (padded coordinates; one more row for B_opt slots), only move down:
 // each lane keeps those rows of its column in registers, adds the point's taps
@@ -48,21 +37,19 @@ __host__ __device__ constexpr size_t spread2d_slot_bytes() {
 // point starts lower it stores the rows that no later point can reach.  Every padded
 // cell is stored exactly once, no shared-memory read-modify-write, no atomics.
 // Window values are computed once per point while staging 32 points per warp.  With PF
-// (window modes: the paired form, and grids too small to hide load latency) the sorted
+// (window modes on grids too small to hide load latency) the sorted
 // data of the next 32 points (perm, cell, u, w) are copied to shared memory with cp.async
 // while the current ones are spread, so that staging waits only on the gather of the
 // samples f.
 // One warp spreads work item gitem (global over the JobSet's jobs); `base` is the warp's
-// shared memory.  The body of k_spread2d, and the spread units of the persistent d = 2 kernel.
+// shared memory.
 template <class R, int MM, bool BOPT, bool PF>
 __device__ __forceinline__ void spread2d_item(const JobSet<R>& js, const int gitem, unsigned char* base) {
     constexpr int W = 2 * MM + 1;              // window taps per axis
-    constexpr int WE = spread2d_we<R, MM, BOPT>();   // stride of the staged rows
+    constexpr int WE = W + 1;                  // stride of the staged rows
     constexpr int WR = BOPT ? W + 1 : W;       // rows held in registers
     constexpr bool F32 = sizeof(R) == 4;
-    constexpr bool PAIR = spread2d_pair<R, MM, BOPT>();
-    constexpr int PX = spread2d_pitch<R, MM, BOPT>();
-    constexpr int NC = PAIR ? 2 : 1;           // columns per lane
+    constexpr int PX = SPREAD2D_PX;
     const int lane = threadIdx.x & 31;
     const int jb = find_job(js.pre_items, js.njobs, gitem);
     const Job<R>& J = js.job[jb];
@@ -81,43 +68,23 @@ __device__ __forceinline__ void spread2d_item(const JobSet<R>& js, const int git
     R* psx = reinterpret_cast<R*>(cy + 32 * WE);            // [32][PX] psi_x by column
     int* meta = reinterpret_cast<int*>(psx + 32 * PX);      // [32][3]  oy, ox, sorted index
     cx<R>* cst = reinterpret_cast<cx<R>*>(meta + 96);       // [32]     c_j (B_opt mode)
-    float* poly = reinterpret_cast<float*>(cst + 32);       // [(WPOLY_DEG+1) * WP] window polynomial (16-byte rows)
-    // the paired form evaluates the taps from the parameter block when every job shares one
-    // window polynomial (js.wtab_ok), else from a copy in shared memory
-    const bool tab_param = PAIR && js.wtab_ok;
-    const bool use_poly = F32 && !BOPT && J.wpoly != nullptr;
-    if (use_poly && !tab_param) {
-        for (int e = lane; e < (WPOLY_DEG + 1) * wpoly_stride(W); e += 32) poly[e] = J.wpoly[e];
-    }
-
     const int ty = item.x / J.ntile, tx = item.x % J.ntile;
     using V2 = typename std::conditional<F32, float2, double2>::type;
-    // (re, im) of the rows r0 .. r0 + WR - 1 of this lane's columns: acc[NC k + c] is row
-    // r0 + k of the lane's column c
-    V2 acc[NC * WR];
+    // (re, im) of the rows r0 .. r0 + WR - 1 of this lane's column
+    V2 acc[WR];
 #pragma unroll
-    for (int k = 0; k < NC * WR; ++k) { acc[k].x = R(0); acc[k].y = R(0); }
-    int r0 = 0;  // padded row held in acc[0 .. NC - 1]
+    for (int k = 0; k < WR; ++k) { acc[k].x = R(0); acc[k].y = R(0); }
+    int r0 = 0;  // padded row held in acc[0]
     int old_ox = -1;   // first column of this lane's taps in its psi_x row, -1: row not zeroed yet
     cx<R>* dst = J.padded + (size_t)it * P * P;
     const bool col_ok = lane < P;
     // store row r0 (no later point reaches it) and move the held rows up by one
     auto flush_row = [&]() {
-        if constexpr (PAIR) {
-            float4 v = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
-            v.x += __shfl_xor_sync(0xffffffffu, v.x, 16);
-            v.y += __shfl_xor_sync(0xffffffffu, v.y, 16);
-            v.z += __shfl_xor_sync(0xffffffffu, v.z, 16);
-            v.w += __shfl_xor_sync(0xffffffffu, v.w, 16);
-            // P and the item's base are even: the column pair is 16-byte aligned
-            if (lane < 16 && 2 * lane < P) *reinterpret_cast<float4*>(dst + (size_t)r0 * P + 2 * lane) = v;
-        } else {
-            if (col_ok) dst[(size_t)r0 * P + lane] = mk<R>(acc[0].x, acc[0].y);
-        }
+        if (col_ok) dst[(size_t)r0 * P + lane] = mk<R>(acc[0].x, acc[0].y);
 #pragma unroll
-        for (int k = 0; k < NC * (WR - 1); ++k) acc[k] = acc[k + NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) { acc[NC * (WR - 1) + c].x = R(0); acc[NC * (WR - 1) + c].y = R(0); }
+        for (int k = 0; k < WR - 1; ++k) acc[k] = acc[k + 1];
+        acc[WR - 1].x = R(0);
+        acc[WR - 1].y = R(0);
         ++r0;
     };
     const int logMs = 31 - __clz(Ms);
@@ -156,22 +123,10 @@ __device__ __forceinline__ void spread2d_item(const JobSet<R>& js, const int git
                 const R uy = PF ? pf_u[2 * lane + 0] : J.u[(size_t)i * 2 + 0];
                 const R ux = PF ? pf_u[2 * lane + 1] : J.u[(size_t)i * 2 + 1];
                 R wy[W], wx[W];
-                bool done = false;
-                if constexpr (F32) {
-                    if (tab_param) {
-                        poly_taps2<W>(js.wtab, uy, ux, wy, wx);
-                        done = true;
-                    } else if (use_poly) {
-                        poly_taps2<W>(poly, uy, ux, wy, wx);
-                        done = true;
-                    }
-                }
-                if (!done) {
 #pragma unroll
-                    for (int s = 0; s < W; ++s) {
-                        wy[s] = tap_weight<R>(J.window, uy, s, MM, J.inv_m, J.beta);
-                        wx[s] = tap_weight<R>(J.window, ux, s, MM, J.inv_m, J.beta);
-                    }
+                for (int s = 0; s < W; ++s) {
+                    wy[s] = tap_weight<R>(J.window, uy, s, MM, J.inv_m, J.beta);
+                    wx[s] = tap_weight<R>(J.window, ux, s, MM, J.inv_m, J.beta);
                 }
                 R* row = psx + lane * PX;
                 // the row is zero off the taps the lane wrote last time: clear those only
@@ -189,7 +144,6 @@ __device__ __forceinline__ void spread2d_item(const JobSet<R>& js, const int git
                     cy[lane * WE + s] = scale(fv, wy[s]);
                     row[oxl + s] = wx[s];
                 }
-                if (WE > W) cy[lane * WE + W] = mk<R>(0, 0);   // the pad the 16-byte row loads read
             }
         }
         __syncwarp();   // orders every read of the prefetch slots before their refill
@@ -206,34 +160,8 @@ __device__ __forceinline__ void spread2d_item(const JobSet<R>& js, const int git
             // store the rows above oy: no later point reaches them
             while (r0 < oy) flush_row();
             const int q = 32 - __clz(__ballot_sync(0xffffffffu, my_oy == oy));
-            if constexpr (PAIR) {
-                // points p + h of each pair go to half h; at an odd run end the second
-                // half adds zeros (the first point's taps times a zero weight)
-                const int half = lane >> 4, hl = lane & 15;
-#pragma unroll 2
-                for (; p < q; p += 2) {
-                    const int pp = p + half;
-                    const bool act = pp < q;
-                    const int pr = act ? pp : p;
-                    float2 wv = *reinterpret_cast<const float2*>(psx + pr * PX + 2 * hl);
-                    if (!act) wv = make_float2(0.f, 0.f);
-                    const float2 wa = make_float2(wv.x, wv.x), wb = make_float2(wv.y, wv.y);
-                    // one 8-byte broadcast per row: the two halves read two points' rows in
-                    // one wavefront
-                    const float2* cp2 = reinterpret_cast<const float2*>(cy + pr * WE);
-#pragma unroll
-                    for (int k = 0; k < W; ++k) {
-                        const float2 c = cp2[k];
-                        acc[2 * k] = __ffma2_rn(c, wa, acc[2 * k]);
-                        acc[2 * k + 1] = __ffma2_rn(c, wb, acc[2 * k + 1]);
-                    }
-                }
-                p = q;
-                continue;
-            }
-            // float32: four points per unrolled step let the loads of the next points
-            // overlap the current FMAs (0.573 -> 0.506 ms before the runs); float64 keeps
-            // its registers for the accumulators
+            // float32: four points per unrolled step let the loads of the next points overlap the
+            // current FMAs; float64 keeps its registers for the accumulators
             constexpr int UNR = F32 ? 4 : 1;
 #pragma unroll UNR
             for (; p < q; ++p) {
@@ -258,24 +186,11 @@ __device__ __forceinline__ void spread2d_item(const JobSet<R>& js, const int git
                 } else {
                     const R wx = psx[p * PX + lane];
                     const cx<R>* cp = cy + p * WE;
-                    if constexpr (F32) {
-                        // two complex coefficients per 16-byte broadcast load, one packed
-                        // two-wide FMA per row
-                        const float4* cp4 = reinterpret_cast<const float4*>(cp);
-                        const float2 ww = make_float2(wx, wx);
 #pragma unroll
-                        for (int k2 = 0; k2 < WE / 2; ++k2) {
-                            const float4 c = cp4[k2];
-                            acc[2 * k2] = __ffma2_rn(make_float2(c.x, c.y), ww, acc[2 * k2]);
-                            if (2 * k2 + 1 < W) acc[2 * k2 + 1] = __ffma2_rn(make_float2(c.z, c.w), ww, acc[2 * k2 + 1]);
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < W; ++k) {
-                            const cx<R> c = cp[k];
-                            acc[k].x += c.re * wx;
-                            acc[k].y += c.im * wx;
-                        }
+                    for (int k = 0; k < W; ++k) {
+                        const cx<R> c = cp[k];
+                        acc[k].x += c.re * wx;
+                        acc[k].y += c.im * wx;
                     }
                 }
             }
@@ -285,41 +200,44 @@ __device__ __forceinline__ void spread2d_item(const JobSet<R>& js, const int git
     while (r0 < P) flush_row();
 }
 
+// warps per block: two of the tensor-core form, four of the register-row form
+template <class R, bool BOPT>
+constexpr int spread2d_wpb() { return spread2d_mma<R, BOPT>() ? 2 : 4; }
+
 template <class R, int MM, bool BOPT, bool PF>
-// the paired form holds 2 (2m + 1) complex accumulators: at most 96 registers, so five 4-warp
-// blocks (20 warps) share an SM (the one-point form ran six at 80 registers)
-__global__ void __launch_bounds__(128, spread2d_pair<R, MM, BOPT>() ? 5 : 1)
+__global__ void __launch_bounds__(32 * spread2d_wpb<R, BOPT>(), spread2d_mma<R, BOPT>() ? (MM <= 4 ? 10 : 6) : 1)
     k_spread2d(const __grid_constant__ JobSet<R> js) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5;
     const int gitem = blockIdx.x * js.wpb + warp;
     if (gitem >= js.pre_items[js.njobs]) return;
-    spread2d_item<R, MM, BOPT, PF>(js, gitem, smem_raw + (size_t)warp * js.smem_per_warp);
+    unsigned char* base = smem_raw + (size_t)warp * js.smem_per_warp;
+    if constexpr (spread2d_mma<R, BOPT>()) spread2d_mma_item<MM>(js, gitem, base);
+    else spread2d_item<R, MM, BOPT, PF>(js, gitem, base);
 }
 
-// Per-launch setup of the register-row spread: shared memory per warp (js.smem_per_warp), four
-// warps per block (js.wpb), and the jobs' common window polynomial in the parameter block.
+// Per-launch setup: shared memory per warp (js.smem_per_warp), warps per block (js.wpb), and for
+// the tensor-core form the jobs' common window polynomial in the parameter block.
 template <class R, int MM, bool BOPT, bool PF>
 static void spread2d_setup(JobSet<R>& js) {
     constexpr int W = 2 * MM + 1;
-    constexpr int WE = spread2d_we<R, MM, BOPT>();
-    size_t spw = spread2d_slot_bytes<R, PF>() + 32 * WE * sizeof(cx<R>) + 32 * spread2d_pitch<R, MM, BOPT>() * sizeof(R) + 96 * sizeof(int) + 32 * sizeof(cx<R>) +
-                 (WPOLY_DEG + 1) * wpoly_stride(W) * sizeof(float);
-    // one window polynomial for every job: into the parameter block
+    js.wpb = spread2d_wpb<R, BOPT>();
     js.wtab_ok = 0;
-    if (spread2d_pair<R, MM, BOPT>() && wpoly_stride(W) <= 12) {
-        const size_t n = (size_t)(WPOLY_DEG + 1) * wpoly_stride(W);
+    if (spread2d_mma<R, BOPT>()) {
+        const size_t n = (size_t)WPOLY_ROWS * wpoly_stride(MM);
         bool same = js.job[0].wpoly_h != nullptr;
         for (int j = 1; j < js.njobs && same; ++j)
             same = js.job[j].wpoly_h && memcmp(js.job[j].wpoly_h, js.job[0].wpoly_h, n * sizeof(float)) == 0;
         if (same) {
-            memcpy(js.wtab, js.job[0].wpoly_h, n * sizeof(float));
+            for (size_t k = 0; k < n; ++k) js.wtab[k] = js.job[0].wpoly_h[k] * spread_mma_wscale(js.job[0].wexp);
             js.wtab_ok = 1;
         }
+        js.smem_per_warp = (SpreadMma<MM>::BYTES + 15) & ~15;
+        return;
     }
-    spw = (spw + 15) & ~(size_t)15;
-    js.smem_per_warp = (int)spw;
-    js.wpb = 4;
+    const size_t spw = spread2d_slot_bytes<R, PF>() + 32 * (W + 1) * sizeof(cx<R>) + 32 * SPREAD2D_PX * sizeof(R) +
+                       96 * sizeof(int) + 32 * sizeof(cx<R>);
+    js.smem_per_warp = (int)((spw + 15) & ~(size_t)15);
 }
 
 // register-row spreading for d = 2 when every job has the same m (2..8) and P <= 32
@@ -331,6 +249,9 @@ static infft_status launch_spread2d_m(JobSet<R>& js, cudaStream_t st) {
     if (nitems == 0) return INFFT_OK;
     const size_t smem = spw * js.wpb;
     INFFT_CUDA(cudaFuncSetAttribute(k_spread2d<R, MM, BOPT, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (spread2d_mma<R, BOPT>())   // shared memory bounds the warps per SM: ask for all of it
+        INFFT_CUDA(cudaFuncSetAttribute(k_spread2d<R, MM, BOPT, PF>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                        (int)cudaSharedmemCarveoutMaxShared));
     k_spread2d<R, MM, BOPT, PF><<<(nitems + js.wpb - 1) / js.wpb, 32 * js.wpb, smem, st>>>(js);
     INFFT_LAUNCHED();
     return INFFT_OK;
@@ -351,18 +272,17 @@ static infft_status launch_spread2d(JobSet<R>& js, cudaStream_t st, int m) {
 
 static bool aligned(const void* p, size_t a) { return ((uintptr_t)p & (a - 1)) == 0; }
 
-// The paired form (float32, m <= 4) always prefetches (batched d = 2, m = 4: spread 0.389 ->
-// 0.383 ms); the one-point forms prefetch only when there are fewer work items than eight
-// warps per SM (with many items, other warps hide the staging's load latency and the copies
-// cost more than they save: 0.428 -> 0.444 ms for the one-point float32 form).  Either way
-// the copies must be aligned element by element.  INFFT_SPREAD2D_PREFETCH=0 or 1 picks the
+// The float64 window form prefetches only when there are fewer work items than eight warps per SM
+// (with many items, other warps hide the staging's load latency and the copies cost more than
+// they save); the tensor-core form loads the next points into registers and has no such choice.
+// The copies must be aligned element by element.  INFFT_SPREAD2D_PREFETCH=0 or 1 picks the
 // form regardless (both give the same sums in the same order).
 template <class R>
-static bool spread2d_prefetch(const JobSet<R>& js, int m) {
+static bool spread2d_prefetch(const JobSet<R>& js) {
     // the first job's plan tuning (1 on, 2 off) comes first, then the environment
     const int env = js.job[0].prefetch == 1 ? 1 : js.job[0].prefetch == 2 ? 0 : env_form("INFFT_SPREAD2D_PREFETCH");
     if (env == 0) return false;
-    if (env != 1 && !spread2d_pair_m<R>(m)) {
+    if (env != 1) {
         int dev = 0, nsm = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -392,7 +312,7 @@ static bool spread2d_eligible(const JobSet<R>& js, int* m_out, bool* bopt_out) {
         // B_opt's extra slot): a tuned tile of 8 at m >= 5 (m >= 4 with B_opt) puts some cells
         // in three tiles along an axis, which the generic path handles
         if (J.P > 2 * J.T) return false;
-        if (!bopt && spread2d_pair_m<R>(m) && (J.P & 1)) return false;   // paired rows: 16-byte stores
+        if (spread2d_mma<R, false>() && !bopt && (J.P & 1)) return false;   // 16-byte stores of column pairs
     }
     if (m < 2 || m > 8) return false;   // m = 8 with window taps only: P = 16 + 16 <= 32
     *m_out = m;
@@ -408,8 +328,10 @@ infft_status spread2d_try(JobSet<R>& js, cudaStream_t st, bool* used) {
     if (!spread2d_eligible(js, &m, &bopt)) return INFFT_OK;
     *used = true;
     if (bopt) return launch_spread2d<R, true, false>(js, st, m);
-    return spread2d_prefetch(js, m) ? launch_spread2d<R, false, true>(js, st, m)
-                                 : launch_spread2d<R, false, false>(js, st, m);
+    if constexpr (!spread2d_mma<R, false>()) {
+        if (spread2d_prefetch(js)) return launch_spread2d<R, false, true>(js, st, m);
+    }
+    return launch_spread2d<R, false, false>(js, st, m);
 }
 
 }  // namespace infft

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(64) k_spread3d(const __grid_constant__ JobSet<
     float* poly = reinterpret_cast<float*>(meta + CH);                 // window polynomial (float32 plans)
     const bool use_poly = F32 && J.wpoly != nullptr;
     if (use_poly) {
-        for (int e = lane; e < (WPOLY_DEG + 1) * wpoly_stride(W); e += 32) poly[e] = J.wpoly[e];
+        for (int e = lane; e < WPOLY_ROWS * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
     }
     for (int e = lane; e < SC; e += 32) { pad[e].x = R(0); pad[e].y = R(0); }
 
@@ -128,29 +128,29 @@ __global__ void __launch_bounds__(64) k_spread3d(const __grid_constant__ JobSet<
             const R uz = PF ? pf_u[3 * lane + 0] : J.u[(size_t)i * 3 + 0];
             const R uy = PF ? pf_u[3 * lane + 1] : J.u[(size_t)i * 3 + 1];
             const R ux = PF ? pf_u[3 * lane + 2] : J.u[(size_t)i * 3 + 2];
-            R wz[W], wy[W], wx[W];
+            R wt[3][W];   // z, y, x
             bool done = false;
             if constexpr (F32) {
                 if (use_poly) {
-                    poly_taps2<W>(poly, uz, uy, wz, wy);
-                    poly_taps<W>(poly, ux, wx);
+                    const float uu[3] = {uz, uy, ux};
+                    poly_taps<MM, 3>(poly, uu, wt);
                     done = true;
                 }
             }
             if (!done) {
 #pragma unroll
                 for (int s = 0; s < W; ++s) {
-                    wz[s] = tap_weight<R>(J.window, uz, s, MM, J.inv_m, J.beta);
-                    wy[s] = tap_weight<R>(J.window, uy, s, MM, J.inv_m, J.beta);
-                    wx[s] = tap_weight<R>(J.window, ux, s, MM, J.inv_m, J.beta);
+                    wt[0][s] = tap_weight<R>(J.window, uz, s, MM, J.inv_m, J.beta);
+                    wt[1][s] = tap_weight<R>(J.window, uy, s, MM, J.inv_m, J.beta);
+                    wt[2][s] = tap_weight<R>(J.window, ux, s, MM, J.inv_m, J.beta);
                 }
             }
 #pragma unroll
             for (int s = 0; s < W; ++s) {
-                cyv[lane * WE + s].x = fv.re * wy[s];
-                cyv[lane * WE + s].y = fv.im * wy[s];
-                psz[lane * WE + s] = wz[s];
-                psx[lane * WE + s] = wx[s];
+                cyv[lane * WE + s].x = fv.re * wt[1][s];
+                cyv[lane * WE + s].y = fv.im * wt[1][s];
+                psz[lane * WE + s] = wt[0][s];
+                psx[lane * WE + s] = wt[2][s];
             }
         }
         __syncwarp();   // orders every read of the prefetch slots before their refill
@@ -216,7 +216,7 @@ static infft_status launch_spread3d_m(JobSet<R>& js, cudaStream_t st) {
     constexpr int CH = spread3d_chunk<R, MM>();
     size_t spw = spread3d_slot_bytes<R, MM, PF>() +
                  ((cells + 1) & ~(size_t)1) * sizeof(cx<R>) + CH * WE * (sizeof(cx<R>) + 2 * sizeof(R)) +
-                 CH * sizeof(int) + (WPOLY_DEG + 1) * wpoly_stride(W) * sizeof(float);
+                 CH * sizeof(int) + WPOLY_ROWS * wpoly_stride(MM) * sizeof(float);
     spw = (spw + 15) & ~(size_t)15;
     const size_t smem_cap = 200 * 1024;
     if (spw > smem_cap) {
