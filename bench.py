@@ -437,7 +437,7 @@ def run_ours(args, rank, world, dist):
     spread_flops = Ntot * ((2 * 4 + 1) ** 2 * 4 + 2 * (2 * 4 + 1) * 2 * 10)
     peak, peak_kind = measured_peak()
     achieved = spread_bytes / (spread_ms / 1e3) / 1e9
-    spread_kernel = "k_spread2d<float, 4, 0, 0>"   # the tensor-core form
+    spread_kernel = "k_spread2d<float, 4, 0>"   # the tensor-core form
     prof = profiled(kernel=spread_kernel)
     # merge and the two FFT passes: bytes of the tensors they read and write (the padded
     # tiles as written by the spread), against their event-timed stage

@@ -233,11 +233,9 @@ infft_status infft_get_bopt(infft_plan_t plan, void* coeff, void* stream);
  *   mode = INFFT_MODE_BOPT : Algorithm 4.4, h = D^* F^* B_opt^* f (needs B_opt).
  *   f    : N complex samples (host or device), caller's point order.
  *   fhat : M^d complex result (host or device), C order over I_M.
- * The spreading kernels for d = 3, and those for d = 2 in float64 on grids with fewer work
- * items than eight warps per SM, copy the next points' sorted data to shared memory while they
- * spread the current ones (the float32 form for d = 2, on the tensor cores, loads them into
- * registers and has no such choice).  INFFT_SPREAD2D_PREFETCH and
- * INFFT_SPREAD3D_PREFETCH in the environment ("0" off, "1" on) override that choice; the
+ * The spreading kernel for d = 3 copies the next points' sorted data to shared memory while it
+ * spreads the current ones (those for d = 2 load them into registers and have no such choice).
+ * INFFT_SPREAD3D_PREFETCH in the environment ("0" off, "1" on) overrides that choice; the
  * sums and their order, and so the results bit for bit, are the same either way.  So with
  * INFFT_FFT_MERGE (on unless "0"): for d = 2 the first FFT pass sums each grid cell from the
  * padded tiles as it loads its rows (steps 2-3 of Algorithm 2.4 with no grid written in

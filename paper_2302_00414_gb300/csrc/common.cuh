@@ -162,6 +162,62 @@ __device__ __forceinline__ void poly_taps(const float* __restrict__ c, const flo
     }
 }
 
+// Float64 plans: the same polynomials of degree 21 (from values to twice the precision, made on the host at
+// plan creation), which reach the rounding level of float64 for any oversampling: the window over one cell
+// varies no faster than exp(pi v), whose Chebyshev coefficients fall below 2e-17 there.  A tap costs 11
+// multiply-adds; the double Bessel function cost several times that, at 1/32 of the float32 rate.
+constexpr int WPOLY64_DEG = 21;
+constexpr int WPOLY64_ROWS = WPOLY64_DEG + 1;
+
+template <class R>
+__host__ __device__ constexpr int wpoly_rows() { return sizeof(R) == 4 ? WPOLY_ROWS : WPOLY64_ROWS; }
+
+template <int MM, int NC>
+__device__ __forceinline__ void poly_taps(const double* __restrict__ c, const double* u, double (*out)[2 * MM + 1]) {
+    constexpr int WP = wpoly_stride(MM);
+#pragma unroll
+    for (int a = 0; a < NC; ++a) {
+        const double v = 2.0 * u[a] - 1.0, v2 = v * v;
+        double ev[MM], od[MM];
+#pragma unroll
+        for (int k = WPOLY64_DEG; k >= 0; --k) {
+#pragma unroll
+            for (int s = 0; s < MM; ++s) {
+                double* p = (k & 1) ? od : ev;
+                p[s] = k >= WPOLY64_DEG - 1 ? c[k * WP + s] : fma(p[s], v2, c[k * WP + s]);
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < MM; ++s) {
+            out[a][s + 1] = fma(od[s], v, ev[s]);
+            out[a][2 * MM - s] = fma(od[s], -v, ev[s]);
+        }
+        out[a][0] = (u[a] == 0.0) ? 1.0 : 0.0;
+    }
+}
+
+// the 2m + 1 taps for m known at run time only
+template <class R>
+__device__ __forceinline__ void poly_taps_any(const R* __restrict__ c, int m, R u, R* out) {
+    const int WP = wpoly_stride(m);
+    constexpr int DEG = sizeof(R) == 4 ? WPOLY_DEG : WPOLY64_DEG;
+    const R v = R(2) * u - R(1), v2 = v * v;
+#pragma unroll 4
+    for (int s = 0; s < m; ++s) {
+        R ev = R(0), od = R(0);
+#pragma unroll
+        for (int k = DEG; k >= 0; --k) {
+            R& p = (k & 1) ? od : ev;
+            const bool low = sizeof(R) == 4 && k == 0;   // float32: c[0]'s low part first
+            p = fma(p, v2, __ldg(c + (low ? DEG + 1 : k) * WP + s));
+            if (low) p += __ldg(c + s);
+        }
+        out[s + 1] = fma(od, v, ev);
+        out[2 * m - s] = fma(od, -v, ev);
+    }
+    out[0] = (u == R(0)) ? R(1) : R(0);
+}
+
 // ----------------------------------------------------------------------------------------
 // Work descriptors.  One Job describes one transform (one plan, one in/out pair);
 // kernels receive an array of Jobs with the same d and precision and map their
@@ -184,7 +240,7 @@ struct Job {
     const int4* items;         // (tile, start, count, 0)
     const int* tile_items;     // ntile^d + 1 prefix of items per tile
     const R* dinv;             // M entries 1/(Ms w^(k)) (per axis); float32: then their low parts
-    const float* wpoly;        // WPOLY_ROWS x wpoly_stride(m) window polynomial (float32 KB plans) or null
+    const R* wpoly;            // wpoly_rows x wpoly_stride(m) window polynomial (Kaiser-Bessel plans) or null
     const float* wpoly_h;      // host copy of the same table (read by the launchers only) or null
     const cx<R>* tw;           // Ms/2 twiddles exp(-2 pi i k / Ms); float32: then their low parts
     cx<R>* padded;             // nitems * P^d

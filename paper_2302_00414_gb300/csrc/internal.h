@@ -38,8 +38,8 @@ struct infft_plan_s {
     void* dinv = nullptr;     // M entries
     void* tw = nullptr;       // Ms/2 complex
     void* dinv_win = nullptr; // M entries for the B_opt window (may alias dinv)
-    float* wpoly = nullptr;   // window polynomial table (float32 Kaiser-Bessel plans)
-    std::vector<float> wpoly_host;   // host copy of that table
+    void* wpoly = nullptr;    // window polynomial table (Kaiser-Bessel plans, plan precision)
+    std::vector<float> wpoly_host;   // host copy of the float32 table
 
     // weights (device): caller order float64 master + sorted copy in plan precision
     void* w_master = nullptr; // N complex128, caller order

@@ -12,12 +12,10 @@ namespace infft {
 // Interpolation for d = 2, 3 with a fixed m: one warp per work item; the warp gathers the
 // padded tile of the grid around its tile into shared memory, then every lane sums the
 // W^d taps of one point in separable order (x innermost, then y, then z) and writes f_j
-// in the caller's order.  Window values come from the float32 polynomial or the exact
-// window (float64 plans).
+// in the caller's order.  Window values come from the plan's polynomial.
 template <class R, int D, int MM>
 __global__ void __launch_bounds__(128) k_interp_t(const __grid_constant__ JobSet<R> js) {
     constexpr int W = 2 * MM + 1;
-    constexpr bool F32 = sizeof(R) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gitem = blockIdx.x * js.wpb + warp;
@@ -29,10 +27,10 @@ __global__ void __launch_bounds__(128) k_interp_t(const __grid_constant__ JobSet
     const int cells = D == 3 ? P * P * P : P * P;
     unsigned char* base = smem_raw + (size_t)warp * js.smem_per_warp;
     cx<R>* pad = reinterpret_cast<cx<R>*>(base);
-    float* poly = reinterpret_cast<float*>(pad + ((cells + 1) & ~1));
-    const bool use_poly = F32 && J.wpoly != nullptr;
+    R* poly = reinterpret_cast<R*>(pad + ((cells + 1) & ~1));
+    const bool use_poly = J.wpoly != nullptr;
     if (use_poly) {
-        for (int e = lane; e < WPOLY_ROWS * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
+        for (int e = lane; e < wpoly_rows<R>() * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
     }
     int tz = 0, ty, tx;
     if (D == 3) { tz = item.x / (nt * nt); ty = (item.x / nt) % nt; tx = item.x % nt; }
@@ -60,14 +58,9 @@ __global__ void __launch_bounds__(128) k_interp_t(const __grid_constant__ JobSet
         R uu[D];
 #pragma unroll
         for (int a = 0; a < D; ++a) uu[a] = J.u[(size_t)i * D + a];
-        bool done = false;
-        if constexpr (F32) {
-            if (use_poly) {
-                poly_taps<MM, D>(poly, uu, wt);
-                done = true;
-            }
-        }
-        if (!done) {
+        if (use_poly) {
+            poly_taps<MM, D>(poly, uu, wt);
+        } else {
 #pragma unroll
             for (int s = 0; s < W; ++s)
 #pragma unroll
@@ -106,7 +99,7 @@ static infft_status launch_interp_t(JobSet<R>& js, cudaStream_t st) {
     int P = 0;
     for (int j = 0; j < js.njobs; ++j) P = std::max(P, js.job[j].P);
     const size_t cells = D == 3 ? (size_t)P * P * P : (size_t)P * P;
-    size_t spw = ((cells + 1) & ~(size_t)1) * sizeof(cx<R>) + WPOLY_ROWS * wpoly_stride(MM) * sizeof(float);
+    size_t spw = ((cells + 1) & ~(size_t)1) * sizeof(cx<R>) + wpoly_rows<R>() * wpoly_stride(MM) * sizeof(R);
     spw = (spw + 15) & ~(size_t)15;
     const size_t smem_cap = 200 * 1024;
     if (spw > smem_cap) {

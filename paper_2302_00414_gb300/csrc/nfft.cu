@@ -75,8 +75,9 @@ __global__ void __launch_bounds__(128) k_spread(const __grid_constant__ JobSet<R
             if (!bopt) {
                 for (int t = 0; t < D; ++t) {
                     const R u = J.u[(size_t)i * D + t];
-                    for (int s = 0; s < W; ++s)
-                        psi[(lane * D + t) * W + s] = tap_weight<R>(J.window, u, s, m, J.inv_m, J.beta);
+                    R* ps = psi + (lane * D + t) * W;
+                    if (J.wpoly) poly_taps_any<R>(J.wpoly, m, u, ps);
+                    else for (int s = 0; s < W; ++s) ps[s] = tap_weight<R>(J.window, u, s, m, J.inv_m, J.beta);
                 }
             }
         }
@@ -352,7 +353,8 @@ __global__ void __launch_bounds__(128) k_interp(const __grid_constant__ JobSet<R
             if (!bopt) {
                 for (int t = 0; t < D; ++t) {
                     const R u = J.u[(size_t)i * D + t];
-                    for (int s = 0; s < W; ++s) ps[t * W + s] = tap_weight<R>(J.window, u, s, m, J.inv_m, J.beta);
+                    if (J.wpoly) poly_taps_any<R>(J.wpoly, m, u, ps + t * W);
+                    else for (int s = 0; s < W; ++s) ps[t * W + s] = tap_weight<R>(J.window, u, s, m, J.inv_m, J.beta);
                 }
             }
             const cx<R>* cf = bopt ? J.coef + (size_t)i * ntap : nullptr;

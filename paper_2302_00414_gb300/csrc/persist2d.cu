@@ -190,7 +190,7 @@ static void build_queue(const JobSet<float>& js, int lag, PersistQueue& pq) {
 
 template <int MM>
 static infft_status launch_persist2d(JobSet<float>& js, cudaStream_t st) {
-    spread2d_setup<float, MM, false, false>(js);
+    spread2d_setup<float, MM, false>(js);
     const size_t smem = std::max({(size_t)4 * js.smem_per_warp, fft_smem_mrg(js), fft_smem(js)});
     auto kern = k_adjoint2d_persistent<MM>;
     INFFT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -72,10 +72,10 @@ __global__ void __launch_bounds__(64) k_spread3d(const __grid_constant__ JobSet<
     R* psz = reinterpret_cast<R*>(cyv + CH * WE);                      // [CH][WE]
     R* psx = psz + CH * WE;                                            // [CH][WE]
     int* meta = reinterpret_cast<int*>(psx + CH * WE);                 // [CH] base cell in the shared tile
-    float* poly = reinterpret_cast<float*>(meta + CH);                 // window polynomial (float32 plans)
-    const bool use_poly = F32 && J.wpoly != nullptr;
+    R* poly = reinterpret_cast<R*>(meta + CH);                 // window polynomial (float32 plans)
+    const bool use_poly = J.wpoly != nullptr;
     if (use_poly) {
-        for (int e = lane; e < WPOLY_ROWS * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
+        for (int e = lane; e < wpoly_rows<R>() * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
     }
     for (int e = lane; e < SC; e += 32) { pad[e].x = R(0); pad[e].y = R(0); }
 
@@ -129,15 +129,10 @@ __global__ void __launch_bounds__(64) k_spread3d(const __grid_constant__ JobSet<
             const R uy = PF ? pf_u[3 * lane + 1] : J.u[(size_t)i * 3 + 1];
             const R ux = PF ? pf_u[3 * lane + 2] : J.u[(size_t)i * 3 + 2];
             R wt[3][W];   // z, y, x
-            bool done = false;
-            if constexpr (F32) {
-                if (use_poly) {
-                    const float uu[3] = {uz, uy, ux};
-                    poly_taps<MM, 3>(poly, uu, wt);
-                    done = true;
-                }
-            }
-            if (!done) {
+            if (use_poly) {
+                const R uu[3] = {uz, uy, ux};
+                poly_taps<MM, 3>(poly, uu, wt);
+            } else {
 #pragma unroll
                 for (int s = 0; s < W; ++s) {
                     wt[0][s] = tap_weight<R>(J.window, uz, s, MM, J.inv_m, J.beta);
@@ -216,7 +211,7 @@ static infft_status launch_spread3d_m(JobSet<R>& js, cudaStream_t st) {
     constexpr int CH = spread3d_chunk<R, MM>();
     size_t spw = spread3d_slot_bytes<R, MM, PF>() +
                  ((cells + 1) & ~(size_t)1) * sizeof(cx<R>) + CH * WE * (sizeof(cx<R>) + 2 * sizeof(R)) +
-                 CH * sizeof(int) + WPOLY_ROWS * wpoly_stride(MM) * sizeof(float);
+                 CH * sizeof(int) + wpoly_rows<R>() * wpoly_stride(MM) * sizeof(R);
     spw = (spw + 15) & ~(size_t)15;
     const size_t smem_cap = 200 * 1024;
     if (spw > smem_cap) {
