@@ -386,6 +386,94 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
 }
 
 
+// Lines of a circular convolution along the last axis (run_fft_conv): each of the A = Ms^(D-1) lines of M
+// values (k in I_M) is zero-padded, transformed with sign +, multiplied by its line of the spectrum,
+// transformed back with sign - and cropped, without leaving shared memory (as two passes and a product it crossed
+// global memory four times at the full length).  The destination may be the source: a block reads its lines
+// before it writes them.
+template <class R, int D, int NTH>
+__device__ __forceinline__ void fft_conv_block(const JobSet<R>& js, const int lb, unsigned char* smem_raw) {
+    const Job<R>& J = js.job[0];
+    const int n = J.Ms, M = J.M, L = fft_lines(n, (int)sizeof(cx<R>)), ns = fft_stride(n, L);
+    const int logn = 31 - __clz(n), logL = 31 - __clz(L);
+    const int nlines = ipow(n, D - 1), q0 = lb * L;
+    cx<R>* from = reinterpret_cast<cx<R>*>(smem_raw);
+    cx<R>* to = from + L * ns;
+    cx<R>* tws = to + L * ns;
+    for (int k = threadIdx.x; k < (n >> 1); k += NTH) {
+        tws[skew(k)] = J.tw[k];
+        if (sizeof(R) == 4) tws[skew(n >> 1) + 1 + skew(k)] = J.tw[(n >> 1) + k];
+    }
+    __syncthreads();
+    const cx<R>* src = (D == 1 ? J.in : D == 2 ? J.tmp1 : J.tmp2) + (size_t)q0 * M;
+    cx<R>* dst = (D == 1 ? J.out : J.tmp1) + (size_t)q0 * M;
+    const cx<R>* spec = J.coef + (size_t)q0 * n;
+    auto ld_in = [&](int l, int j, int q, auto& v) {
+        constexpr int RX = sizeof(v) / sizeof(v[0]);
+#pragma unroll
+        for (int r = 0; r < RX; ++r) {
+            const int i = (j + r * q + M / 2) & (n - 1);
+            v[r] = (i < M && q0 + l < nlines) ? src[(size_t)l * M + i] : mk<R>(0, 0);
+        }
+    };
+    auto ld_buf = [&](int l, int j, int q, auto& v) {
+        constexpr int RX = sizeof(v) / sizeof(v[0]);
+#pragma unroll
+        for (int r = 0; r < RX; ++r) v[r] = from[l * ns + skew(j + r * q)];
+    };
+    auto st_to = [&](int l, int i, cx<R> v) { to[l * ns + skew(i)] = v; };
+    auto st_spec = [&](int l, int i, cx<R> v) {
+        if (q0 + l < nlines) v = mul(v, spec[(size_t)l * n + i]);
+        to[l * ns + skew(i)] = v;
+    };
+    auto st_out = [&](int l, int i, cx<R> v) {
+        const int k = (i + M / 2) & (n - 1);
+        if (k < M && q0 + l < nlines) dst[(size_t)l * M + k] = v;
+    };
+    auto swap_bufs = [&]() {
+        __syncthreads();
+        cx<R>* const s = from;
+        from = to;
+        to = s;
+    };
+    const int nfour = logn % 3 == 0 ? 0 : logn % 3 == 2 ? 1 : 2, neight = (logn - 2 * nfour) / 3;
+    // forward; the last stage multiplies by the spectrum as it stores
+    int logNs = 0;
+    while (logNs < logn) {
+        const bool eight = logNs < 3 * neight, first = logNs == 0;
+        const int next = logNs + (eight ? 3 : 2);
+        const bool end = next == logn;
+        if (eight) {
+            if (first && end) fft_stage<R, true, 8, NTH>(L, logL, logn, logNs, false, tws, ld_in, st_spec);
+            else if (first) fft_stage<R, true, 8, NTH>(L, logL, logn, logNs, false, tws, ld_in, st_to);
+            else if (end) fft_stage<R, true, 8, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_spec);
+            else fft_stage<R, true, 8, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_to);
+        } else {
+            if (first && end) fft_stage<R, true, 4, NTH>(L, logL, logn, logNs, false, tws, ld_in, st_spec);
+            else if (first) fft_stage<R, true, 4, NTH>(L, logL, logn, logNs, false, tws, ld_in, st_to);
+            else if (end) fft_stage<R, true, 4, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_spec);
+            else fft_stage<R, true, 4, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_to);
+        }
+        swap_bufs();
+        logNs = next;
+    }
+    // and back
+    logNs = 0;
+    while (logNs < logn) {
+        const bool eight = logNs < 3 * neight;
+        const int next = logNs + (eight ? 3 : 2);
+        if (next == logn) {
+            if (eight) fft_stage<R, false, 8, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_out);
+            else fft_stage<R, false, 4, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_out);
+            return;
+        }
+        if (eight) fft_stage<R, false, 8, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_to);
+        else fft_stage<R, false, 4, NTH>(L, logL, logn, logNs, false, tws, ld_buf, st_to);
+        swap_bufs();
+        logNs = next;
+    }
+}
+
 // The halo merge of the d = 2 register-row path folded into the first FFT pass (fft_block with
 // MRG), unless INFFT_FFT_MERGE=0 or a job's table of tile item ranges would pass 16 KB: the
 // grid is then neither written nor read between the two.  Both forms give bitwise the same

@@ -179,6 +179,11 @@ infft_status run_fft_axis(const Job<R>& J, long long A, long long B, int nblk, c
 template <class R>
 infft_status run_fft_passes(const Job<R>& J, cudaStream_t st, bool forward);
 
+// J.out = crop of F^- (J.coef .* F^+ zero-padded J.in): a circular convolution of period Ms per axis with the
+// spectrum J.coef (Ms^d), M^d values in and out; J.tw, J.tmp1, J.tmp2 as for run_fft_passes, J.dinv must be ones.
+template <class R>
+infft_status run_fft_conv(const Job<R>& J, cudaStream_t st);
+
 // bounded waits of the persistent d = 2 kernel that gave up since the library was loaded
 unsigned int persist_wait_timeouts();
 

@@ -294,6 +294,12 @@ __global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? (MRG ? 5 : 
     fft_block<R, D, FWD, MRG, fft_threads<R>()>(js, pass, blockIdx.x, smem_raw);
 }
 
+template <class R, int D>
+__global__ void __launch_bounds__(fft_threads<R>()) k_fft_conv(const __grid_constant__ JobSet<R> js) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fft_conv_block<R, D, fft_threads<R>()>(js, blockIdx.x, smem_raw);
+}
+
 // ---------------------------------------------------------------------------------------
 // interpolation (Algorithm 2.1 step 3): one warp per work item; the warp copies the
 // padded tile of the grid around its tile into shared memory, then every lane sums the
@@ -685,6 +691,42 @@ infft_status run_fft_passes(const Job<R>& J, cudaStream_t st, bool forward) {
     }
 }
 
+template <class R, int D>
+static infft_status fft_conv_d(const Job<R>& J, cudaStream_t st) {
+    JobSet<R> js, ja;   // prefixes of the forward and of the adjoint passes
+    memset(&js, 0, sizeof(js));
+    js.njobs = 1;
+    js.job[0] = J;
+    ja = js;
+    fill_prefixes(js, D, true);
+    fill_prefixes(ja, D, false);
+    const size_t smem = fft_smem(js);
+    for (int p = 0; p + 1 < D; ++p) {
+        INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_fft<R, D, true><<<js.pre_fft[p][1], fft_threads<R>(), smem, st>>>(js, p);
+        INFFT_LAUNCHED();
+    }
+    INFFT_CUDA(cudaFuncSetAttribute(k_fft_conv<R, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_fft_conv<R, D><<<ja.pre_fft[0][1], fft_threads<R>(), smem, st>>>(ja);
+    INFFT_LAUNCHED();
+    for (int p = 1; p < D; ++p) {
+        INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_fft<R, D, false><<<ja.pre_fft[p][1], fft_threads<R>(), smem, st>>>(ja, p);
+        INFFT_LAUNCHED();
+    }
+    return INFFT_OK;
+}
+
+template <class R>
+infft_status run_fft_conv(const Job<R>& J, cudaStream_t st) {
+    switch (J.d) {
+        case 1: return fft_conv_d<R, 1>(J, st);
+        case 2: return fft_conv_d<R, 2>(J, st);
+        default: return fft_conv_d<R, 3>(J, st);
+    }
+}
+
+template infft_status run_fft_conv<double>(const Job<double>&, cudaStream_t);
 template infft_status run_fft_passes<double>(const Job<double>&, cudaStream_t, bool);
 template infft_status run_jobs<float>(const std::vector<Job<float>>&, cudaStream_t, bool, cudaEvent_t*);
 template infft_status run_jobs<double>(const std::vector<Job<double>>&, cudaStream_t, bool, cudaEvent_t*);

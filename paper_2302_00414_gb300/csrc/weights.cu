@@ -23,49 +23,50 @@
 namespace infft {
 
 
-constexpr int RED_BLOCKS = 1024;
+// two blocks per SM: a fixed grid, so that the sums do not depend on the device's load
+constexpr int RED_BLOCKS = 304;
 constexpr int RED_THREADS = 256;
 
-// partial sums of sum_i conj(a_i) b_i over a fixed grid: deterministic
-__global__ void __launch_bounds__(RED_THREADS) k_dot_partial(const cx<double>* __restrict__ a,
-                                                             const cx<double>* __restrict__ b, long long n,
-                                                             double* __restrict__ part) {
+// A sum over a fixed grid of blocks, finished by the block that ends last: every block stores its partial
+// sum, and the last one (counted by a ticket that wraps to zero for the next use) adds the partial sums in block
+// order.  Deterministic, and one launch where partial and final sum took two.  True in every thread of
+// the last block, with the whole sum in (re, im).
+__device__ bool grid_sum(double& re, double& im, double* part, unsigned* ticket) {
     __shared__ double sre[RED_THREADS], sim[RED_THREADS];
-    double re = 0, im = 0;
-    for (long long i = (long long)blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += (long long)RED_BLOCKS * RED_THREADS) {
-        const cx<double> x = a[i], y = b[i];
-        re += x.re * y.re + x.im * y.im;
-        im += x.re * y.im - x.im * y.re;
-    }
-    sre[threadIdx.x] = re;
-    sim[threadIdx.x] = im;
-    __syncthreads();
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            sre[threadIdx.x] += sre[threadIdx.x + s];
-            sim[threadIdx.x] += sim[threadIdx.x + s];
+    __shared__ bool last;
+    const int t = threadIdx.x;
+    auto block_sum = [&]() {
+        sre[t] = re;
+        sim[t] = im;
+        __syncthreads();
+        for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
+            if (t < s) {
+                sre[t] += sre[t + s];
+                sim[t] += sim[t + s];
+            }
+            __syncthreads();
         }
-        __syncthreads();
+        re = sre[0];
+        im = sim[0];
+    };
+    block_sum();
+    if (t == 0) {
+        part[2 * blockIdx.x] = re;
+        part[2 * blockIdx.x + 1] = im;
+        __threadfence();
+        last = atomicInc(ticket, RED_BLOCKS - 1) == RED_BLOCKS - 1;
     }
-    if (threadIdx.x == 0) {
-        part[2 * blockIdx.x] = sre[0];
-        part[2 * blockIdx.x + 1] = sim[0];
-    }
-}
-
-// out[0..1] = sum of the partials (fixed order)
-__global__ void k_dot_final(const double* __restrict__ part, double* __restrict__ out) {
-    __shared__ double sre[RED_THREADS], sim[RED_THREADS];
-    double re = 0, im = 0;
-    for (int i = threadIdx.x; i < RED_BLOCKS; i += RED_THREADS) { re += part[2 * i]; im += part[2 * i + 1]; }
-    sre[threadIdx.x] = re;
-    sim[threadIdx.x] = im;
     __syncthreads();
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) { sre[threadIdx.x] += sre[threadIdx.x + s]; sim[threadIdx.x] += sim[threadIdx.x + s]; }
-        __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    re = 0;
+    im = 0;
+    for (int i = t; i < RED_BLOCKS; i += RED_THREADS) {
+        re += __ldcg(part + 2 * i);
+        im += __ldcg(part + 2 * i + 1);
     }
-    if (threadIdx.x == 0) { out[0] = sre[0]; out[1] = sim[0]; }
+    block_sum();
+    return true;
 }
 
 // CG scalars, all on the device: s[0] = rr, s[2] = <p, q>, s[4] = rr_new, s[6] = alpha,
@@ -73,15 +74,52 @@ __global__ void k_dot_final(const double* __restrict__ part, double* __restrict_
 // 3 max_iter reached), s[12] = iterations taken, s[13] = (rel_tol ||b||)^2, s[14] = max_iter,
 // s[15] = this iteration improved on s[10], s[16] = this iteration runs.  Every kernel of an
 // iteration is a no-op once the state is no longer 0, so the host may queue several
-// iterations between looks at the state.
-__global__ void k_cg_begin(double* s) { s[16] = (s[11] == 0.0) ? 1.0 : 0.0; }
-__global__ void k_cg_alpha(double* s) {
-    if (s[16] == 0.0) return;
-    s[6] = (s[2] != 0.0) ? s[0] / s[2] : 0.0;
+// iterations between looks at the state.  Three kernels per iteration beside the matrix product
+// (nine before, each a few microseconds of launch and drain).
+
+// s[0] = <a, a>
+__global__ void __launch_bounds__(RED_THREADS) k_cg_norm(const cx<double>* __restrict__ a, long long n,
+                                                         double* __restrict__ part, unsigned* ticket, double* s) {
+    double re = 0, im = 0;
+    for (long long i = (long long)blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += (long long)RED_BLOCKS * RED_THREADS)
+        re += a[i].re * a[i].re + a[i].im * a[i].im;
+    if (grid_sum(re, im, part, ticket) && threadIdx.x == 0) s[0] = re;
 }
-__global__ void k_cg_end(double* s) {
+
+// alpha = rr / <p, q>
+__global__ void __launch_bounds__(RED_THREADS) k_cg_alpha(const cx<double>* __restrict__ p,
+                                                          const cx<double>* __restrict__ q, long long n,
+                                                          double* __restrict__ part, unsigned* ticket, double* s) {
+    double re = 0, im = 0;
+    for (long long i = (long long)blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += (long long)RED_BLOCKS * RED_THREADS) {
+        const cx<double> x = p[i], y = q[i];
+        re += x.re * y.re + x.im * y.im;
+        im += x.re * y.im - x.im * y.re;
+    }
+    if (!grid_sum(re, im, part, ticket) || threadIdx.x != 0) return;
+    s[16] = (s[11] == 0.0) ? 1.0 : 0.0;
     if (s[16] == 0.0) return;
-    const double rn = s[4];
+    s[2] = re;
+    s[6] = (re != 0.0) ? s[0] / re : 0.0;
+}
+
+// x += alpha p, r -= alpha q, then the iteration's residual, best iterate, beta and state
+__global__ void __launch_bounds__(RED_THREADS) k_cg_update_xr(cx<double>* __restrict__ x, cx<double>* __restrict__ r,
+                                                              const cx<double>* __restrict__ p,
+                                                              const cx<double>* __restrict__ q, long long n,
+                                                              double* __restrict__ part, unsigned* ticket, double* s) {
+    if (s[16] == 0.0) return;
+    const double al = s[6];
+    double re = 0, im = 0;
+    for (long long i = (long long)blockIdx.x * RED_THREADS + threadIdx.x; i < n; i += (long long)RED_BLOCKS * RED_THREADS) {
+        x[i] = add(x[i], scale(p[i], al));
+        const cx<double> v = sub(r[i], scale(q[i], al));
+        r[i] = v;
+        re += v.re * v.re + v.im * v.im;
+    }
+    if (!grid_sum(re, im, part, ticket) || threadIdx.x != 0) return;
+    const double rn = re;
+    s[4] = rn;
     s[12] += 1.0;
     if (!(rn == rn)) { s[11] = 2.0; s[15] = 0.0; return; }
     s[15] = (rn < s[10]) ? 1.0 : 0.0;
@@ -92,32 +130,18 @@ __global__ void k_cg_end(double* s) {
     else if (s[12] >= s[14]) s[11] = 3.0;
 }
 
-__global__ void k_cg_update_xr(cx<double>* __restrict__ x, cx<double>* __restrict__ r, const cx<double>* __restrict__ p,
-                               const cx<double>* __restrict__ q, long long n, const double* __restrict__ s) {
-    if (s[16] == 0.0) return;
-    const double al = s[6];
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        x[i] = add(x[i], scale(p[i], al));
-        r[i] = sub(r[i], scale(q[i], al));
-    }
-}
-
 // x_best = x when this iteration's residual is the smallest so far (the weights come from
 // the best iterate, so that a capped CG never returns worse weights than an earlier step of
-// the same run)
-__global__ void k_cg_keep_best(const cx<double>* __restrict__ x, cx<double>* __restrict__ xb, long long n,
-                               const double* __restrict__ s) {
-    if (s[16] == 0.0 || s[15] == 0.0) return;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        xb[i] = x[i];
-}
-
-__global__ void k_cg_update_p(cx<double>* __restrict__ p, const cx<double>* __restrict__ r, long long n,
-                              const double* __restrict__ s) {
-    if (s[16] == 0.0 || s[11] != 0.0) return;
+// the same run); p = r + beta p while the CG goes on
+__global__ void k_cg_next(const cx<double>* __restrict__ x, cx<double>* __restrict__ xb, cx<double>* __restrict__ p,
+                          const cx<double>* __restrict__ r, long long n, const double* __restrict__ s) {
+    if (s[16] == 0.0) return;
+    const bool keep = s[15] != 0.0, on = s[11] == 0.0;
     const double be = s[7];
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        p[i] = add(r[i], scale(p[i], be));
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        if (keep) xb[i] = x[i];
+        if (on) p[i] = add(r[i], scale(p[i], be));
+    }
 }
 
 // the CG's starting scalars: rr = ||b||^2, no best iterate yet (the first iteration always
@@ -200,11 +224,12 @@ __global__ void k_sort_weights(const cx<double>* __restrict__ master, const int*
 // so A^* A u is a d-variate discrete convolution of t with u.  t on I_4M is obtained once
 // from 2^d adjoint NFFTs at degree 2M of modulated unit samples,
 //   t(s + k) = sum_j exp(-2 pi i s x_j) exp(-2 pi i k x_j),  s in {-M, M}^d, k in I_2M,
-// and the convolution is a circular one of period L = 4M (u zero-padded):
+// of which t(-n) = conj(t(n)) needs only those with s_0 = M, and the convolution is a circular one of period L = 4M (u zero-padded):
 //   A^* A u = crop_{I_2M} F_L^- ( c_hat .* F_L^+ u ),  c_hat = L^{-d} F_L^+ t,
 // where F_L^+ / F_L^- are the unnormalised DFTs with sign + / - (the pruned FFT passes with
 // unit deconvolution factors).  Each CG iteration is then two FFTs of L^d points instead of
-// an NFFT and an adjoint NFFT.
+// an NFFT and an adjoint NFFT; the last axis' transform, the product and the transform back are one pass
+// over lines held in shared memory (run_fft_conv).
 
 // f_j = exp(-2 pi i sum_t s_t x_{j,t}), s_t = -M2/2 or +M2/2 by bit t of `bits`; each
 // s_t x_t is exact (M2/2 is a power of two) and is reduced mod 1 before the sum
@@ -222,26 +247,27 @@ __global__ void k_modulate(const double* __restrict__ x, int N, int d, int M2, i
     f[j] = mk<double>(cs, sn);
 }
 
-// place the degree-2M result of shift `bits` into I_4M: entry (i_t)_t of h goes to
-// (i_t + M2 bit_t)_t of t (C order, 2 M2 per axis)
+// place the degree-2M result of shift `bits` (bit 0 set: n_0 = 0..M2-1) into I_4M: entry (i_t)_t of h is
+// t(n) with n_t = i_t - M2 (1 - bit_t), stored at n_t + M2 (C order, 2 M2 per axis).  t is the transform of real
+// samples, t(-n) = conj(t(n)), which gives the entries with n_0 < 0 (but for those with some n_t = -M2, which no
+// difference k - k' reaches: they stay zero).
 __global__ void k_scatter_t(const cx<double>* __restrict__ h, int d, int M2, int bits, cx<double>* __restrict__ t) {
     long long K = 1;
     for (int q = 0; q < d; ++q) K *= M2;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= K) return;
-    long long rem = i, dst = 0, stride = 1;
+    long long rem = i, dst = 0, mir = 0, stride = 1;
+    bool mirror = true;
     for (int q = d - 1; q >= 0; --q) {
-        const int it = (int)(rem % M2);
+        const int n = (int)(rem % M2) - (((bits >> q) & 1) ? 0 : M2);
         rem /= M2;
-        dst += (long long)(it + (((bits >> q) & 1) ? M2 : 0)) * stride;
+        dst += (long long)(M2 + n) * stride;
+        mir += (long long)(M2 - n) * stride;
         stride *= 2LL * M2;
+        mirror = mirror && n > -M2 && (q > 0 || n > 0);
     }
     t[dst] = h[i];
-}
-
-__global__ void k_cmul(cx<double>* __restrict__ a, const cx<double>* __restrict__ b, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        a[i] = mul(a[i], b[i]);
+    if (mirror) t[mir] = conjg(h[i]);
 }
 
 __global__ void k_fill_real(double* __restrict__ a, int n, double v) {
@@ -259,11 +285,7 @@ __global__ void k_twiddles(int L, cx<double>* __restrict__ tw) {
 }
 
 struct ToeplitzOp {
-    Job<double> fwd;     // u (I_2M) -> G (L^d), sign +
-    Job<double> adj;     // G -> A^*A u (I_2M), sign -
-    cx<double>* G = nullptr;
-    const cx<double>* chat = nullptr;
-    long long Ld = 0;
+    Job<double> job;     // u (I_2M) -> A^*A u, coef = c_hat
 };
 
 static infft_status nfft64(infft_plan_s* q, bool forward, const void* in, void* out, cudaStream_t st);
@@ -294,7 +316,8 @@ static infft_status toeplitz_setup(const infft_plan_s* p, infft_plan_s* sub, int
     k_fill_real<<<(L + 255) / 256, 256, 0, st>>>(invL, L, 1.0 / L);
     INFFT_LAUNCHED();
     // t on I_4M, stored in G
-    for (int bits = 0; bits < (1 << d); ++bits) {
+    INFFT_CUDA(cudaMemsetAsync(G, 0, Ld * 16, st));
+    for (int bits = 1; bits < (1 << d); bits += 2) {
         k_modulate<<<(N + 255) / 256, 256, 0, st>>>(p->x64, N, d, M2, bits, fm);
         INFFT_LAUNCHED();
         INFFT_TRY(nfft64(sub, false, fm, hb, st));
@@ -307,37 +330,23 @@ static infft_status toeplitz_setup(const infft_plan_s* p, infft_plan_s* sub, int
     // c_hat = L^{-d} F_L^+ t: every frequency of I_4M is an input (M = Ms = L)
     J.M = L; J.Ms = L; J.dinv = invL; J.in = G; J.grid = chat;
     INFFT_TRY(run_fft_passes<double>(J, st, true));
-    op.fwd = J;
-    op.fwd.M = M2; op.fwd.dinv = ones; op.fwd.grid = G;
-    op.adj = op.fwd;
-    op.G = G;
-    op.chat = chat;
-    op.Ld = Ld;
+    op.job = J;
+    op.job.M = M2;
+    op.job.dinv = ones;
+    op.job.coef = chat;
     return INFFT_OK;
 }
 
 // q = A^* A p through the Toeplitz operator
 static infft_status toeplitz_apply(ToeplitzOp& op, const cx<double>* pin, cx<double>* qout, cudaStream_t st) {
-    op.fwd.in = pin;
-    INFFT_TRY(run_fft_passes<double>(op.fwd, st, true));
-    k_cmul<<<1024, 256, 0, st>>>(op.G, op.chat, op.Ld);
-    INFFT_LAUNCHED();
-    op.adj.out = qout;
-    return run_fft_passes<double>(op.adj, st, false);
+    op.job.in = pin;
+    op.job.out = qout;
+    return run_fft_conv<double>(op.job, st);
 }
 
 static infft_status nfft64(infft_plan_s* q, bool forward, const void* in, void* out, cudaStream_t st) {
     std::vector<Job<double>> jobs{make_job<double>(q, INFFT_MODE_PLAIN, in, out)};
     return run_jobs<double>(jobs, st, forward);
-}
-
-static infft_status dot(const cx<double>* a, const cx<double>* b, long long n, double* part, double* out,
-                        cudaStream_t st) {
-    k_dot_partial<<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, n, part);
-    INFFT_LAUNCHED();
-    k_dot_final<<<1, RED_THREADS, 0, st>>>(part, out);
-    INFFT_LAUNCHED();
-    return INFFT_OK;
 }
 
 static infft_status ensure_weight_buffers(infft_plan_s* p) {
@@ -406,7 +415,10 @@ static infft_status weights_impl(infft_plan_s* p, int max_iter, double rel_tol, 
         INFFT_LAUNCHED();
     }
     INFFT_CUDA(cudaMemcpyAsync(pv, r, n * 16, cudaMemcpyDeviceToDevice, st));
-    INFFT_TRY(dot(r, r, n, part, sc + 0, st));  // rr = ||b||^2
+    unsigned* ticket = reinterpret_cast<unsigned*>(sc + 24);
+    INFFT_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned), st));
+    k_cg_norm<<<RED_BLOCKS, RED_THREADS, 0, st>>>(r, n, part, ticket, sc);  // rr = ||b||^2
+    INFFT_LAUNCHED();
     k_cg_init<<<1, 1, 0, st>>>(sc, rel_tol, max_iter);
     INFFT_LAUNCHED();
 
@@ -418,8 +430,6 @@ static infft_status weights_impl(infft_plan_s* p, int max_iter, double rel_tol, 
     while (queued < max_iter) {
         const int chunk = std::min(8, max_iter - queued);
         for (int c = 0; c < chunk; ++c) {
-            k_cg_begin<<<1, 1, 0, st>>>(sc);
-            INFFT_LAUNCHED();
             // q = op(p)
             if (toeplitz) {
                 INFFT_TRY(toeplitz_apply(top, pv, qv, st));   // A^* A p as a convolution
@@ -430,17 +440,11 @@ static infft_status weights_impl(infft_plan_s* p, int max_iter, double rel_tol, 
                 INFFT_TRY(nfft64(sub, false, pv, aux, st));   // A^* p (N -> K)
                 INFFT_TRY(nfft64(sub, true, aux, qv, st));    // A (A^* p)
             }
-            INFFT_TRY(dot(pv, qv, n, part, sc + 2, st));
-            k_cg_alpha<<<1, 1, 0, st>>>(sc);
+            k_cg_alpha<<<RED_BLOCKS, RED_THREADS, 0, st>>>(pv, qv, n, part, ticket, sc);
             INFFT_LAUNCHED();
-            k_cg_update_xr<<<eb, et, 0, st>>>(x, r, pv, qv, n, sc);
+            k_cg_update_xr<<<RED_BLOCKS, RED_THREADS, 0, st>>>(x, r, pv, qv, n, part, ticket, sc);
             INFFT_LAUNCHED();
-            INFFT_TRY(dot(r, r, n, part, sc + 4, st));
-            k_cg_end<<<1, 1, 0, st>>>(sc);
-            INFFT_LAUNCHED();
-            k_cg_keep_best<<<eb, et, 0, st>>>(x, xb, n, sc);
-            INFFT_LAUNCHED();
-            k_cg_update_p<<<eb, et, 0, st>>>(pv, r, n, sc);
+            k_cg_next<<<RED_BLOCKS, RED_THREADS, 0, st>>>(x, xb, pv, r, n, sc);
             INFFT_LAUNCHED();
         }
         queued += chunk;
