@@ -126,8 +126,8 @@ static bool interp_t_eligible(const JobSet<R>& js, int* m_out) {
         const Job<R>& J = js.job[j];
         if (J.m != m || J.mode == INFFT_MODE_BOPT || (J.T & (J.T - 1)) != 0 || (J.Ms & (J.Ms - 1)) != 0) return false;
     }
-    // float64 d = 2 up to the CG's m = 8; otherwise m <= 6
-    if (m < 1 || m > ((D == 2 && sizeof(R) == 8) ? 8 : 6)) return false;
+    // d = 2 up to the CG's m = 8; d = 3 up to 6
+    if (m < 1 || m > (D == 2 ? 8 : 6)) return false;
     *m_out = m;
     return true;
 }
@@ -142,7 +142,7 @@ static infft_status launch_interp(JobSet<R>& js, cudaStream_t st, int m) {
         case 5: return launch_interp_t<R, D, 5>(js, st);
         case 6: return launch_interp_t<R, D, 6>(js, st);
         default:
-            if constexpr (D == 2 && sizeof(R) == 8) {
+            if constexpr (D == 2) {
                 if (m == 7) return launch_interp_t<R, D, 7>(js, st);
                 return launch_interp_t<R, D, 8>(js, st);
             }

@@ -11,6 +11,13 @@
 
 namespace infft {
 
+// the slots of a point on the lanes of a warp: 16-byte loads of VEC coefficients, NR per lane; off(r) is the first
+// one's cell relative to the point's first cell in a tile of row length P
+template <class R, int MM>
+struct BoptLanes {
+    static constexpr int S = 2 * MM + 2, VEC = 16 / (int)sizeof(cx<R>), NV = S * S / VEC, NR = (NV + 31) / 32;
+};
+
 // cp.async of one aligned element of B bytes (4, 8 or 16) from global to shared memory
 template <int B>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem) {

@@ -16,123 +16,125 @@ namespace infft {
 // Window modes: float32 takes the tensor-core form of spreadmma.cuh, float64 the form of spread64.cuh.
 
 // ---------------------------------------------------------------------------------------
-// Two-dimensional spreading with B_opt, the accumulators in registers.  One warp per work
-// item; lane l owns column l of the item's P x P padded tile (P = T + 2m + 1 <= 32).
-// The item's points are sorted by base row, so the rows a point can touch,
-// [oy, oy + 2m + 1] (padded coordinates), only move down: each lane keeps those rows of its
-// column in registers, adds the point's coefficients of its column (conjugated) times the sample,
-// and when the next point starts lower it stores the rows that no later point can reach.  Every padded
-// cell is stored exactly once, no shared-memory read-modify-write, no atomics.
-// One warp spreads work item gitem (global over the JobSet's jobs); `base` is the warp's
-// shared memory.
+// Two-dimensional spreading with B_opt (Algorithm 4.4).  A point's S x S coefficients (S = 2m + 2)
+// are one contiguous run of memory, and reading them is what this kernel has to do.  Four warps share a work
+// item, each taking a quarter of its points in order; a warp's lanes take the point's coefficients 16 bytes
+// each, whole runs at a time (a lane per padded column read ten strided rows of 80 bytes), four
+// points' loads in flight before the first is used, and add conj(b) f to the warp's own padded tile in
+// shared memory.  The four tiles are summed in warp order, so that the order of every sum is fixed.
+constexpr int SPREAD_BOPT_WARPS = 4;
+
 template <class R, int MM>
-__device__ __forceinline__ void spread2d_bopt_item(const JobSet<R>& js, const int gitem, unsigned char* base) {
-    constexpr int S = 2 * MM + 2;              // slots per axis, and rows held in registers
-    constexpr bool F32 = sizeof(R) == 4;
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void spread2d_bopt_item(const JobSet<R>& js, const int gitem, unsigned char* smem) {
+    using C = BoptLanes<R, MM>;
+    constexpr int VEC = C::VEC, NV = C::NV, NR = C::NR, S = C::S, NW = SPREAD_BOPT_WARPS;
+    using V = typename std::conditional<sizeof(R) == 4, float4, double2>::type;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int jb = find_job(js.pre_items, js.njobs, gitem);
     const Job<R>& J = js.job[jb];
     const int it = gitem - js.pre_items[jb];
     const int4 item = J.items[it];
-    const int P = J.P, Ms = J.Ms, T = J.T;
-    cx<R>* cst = reinterpret_cast<cx<R>*>(base);            // [32]     c_j
-    int* meta = reinterpret_cast<int*>(cst + 32);           // [32][3]  oy, ox, sorted index
+    const int P = J.P, Ms = J.Ms, T = J.T, cells = P * P;
     const int ty = item.x / J.ntile, tx = item.x % J.ntile;
-    using V2 = typename std::conditional<F32, float2, double2>::type;
-    // (re, im) of the rows r0 .. r0 + S - 1 of this lane's column
-    V2 acc[S];
-#pragma unroll
-    for (int k = 0; k < S; ++k) { acc[k].x = R(0); acc[k].y = R(0); }
-    int r0 = 0;  // padded row held in acc[0]
-    cx<R>* dst = J.padded + (size_t)it * P * P;
-    const bool col_ok = lane < P;
-    // store row r0 (no later point reaches it) and move the held rows up by one
-    auto flush_row = [&]() {
-        if (col_ok) dst[(size_t)r0 * P + lane] = mk<R>(acc[0].x, acc[0].y);
-#pragma unroll
-        for (int k = 0; k < S - 1; ++k) acc[k] = acc[k + 1];
-        acc[S - 1].x = R(0);
-        acc[S - 1].y = R(0);
-        ++r0;
-    };
     const int logMs = 31 - __clz(Ms);
-    for (int c0 = 0; c0 < item.z; c0 += 32) {
-        const int np = min(32, item.z - c0);
-        __syncwarp();
+    cx<R>* pad = reinterpret_cast<cx<R>*>(smem) + warp * cells;
+    for (int e = lane; e < cells; e += 32) pad[e] = mk<R>(0, 0);
+    int off[NR];
+    bool act[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int q = VEC * (lane + 32 * r);
+        act[r] = lane + 32 * r < NV;
+        off[r] = act[r] ? (q / S) * P + q % S : 0;
+    }
+    __syncwarp();
+    const int per = (item.z + NW - 1) / NW, first = min(item.z, warp * per), last = min(item.z, first + per);
+    for (int c0 = first; c0 < last; c0 += 32) {
+        const int np = min(32, last - c0);
+        int o = 0;
+        cx<R> f = mk<R>(0, 0);
         if (lane < np) {
             const int i = item.y + c0 + lane;
             const uint32_t cl = __ldg(J.cell + i);
-            meta[lane * 3 + 0] = (int)(cl >> logMs) - ty * T;
-            meta[lane * 3 + 1] = (int)(cl & (uint32_t)(Ms - 1)) - tx * T;
-            meta[lane * 3 + 2] = i;
-            cst[lane] = J.in[__ldg(J.perm + i)];
+            o = ((int)(cl >> logMs) - ty * T) * P + (int)(cl & (uint32_t)(Ms - 1)) - tx * T;
+            f = J.in[__ldg(J.perm + i)];
         }
-        __syncwarp();
-        // The points are sorted by base row, so the chunk splits into runs of equal oy
-        // (found by one ballot): the rows above a run are stored once per run, and the
-        // points of a run only add their taps.
-        const int my_oy = lane < np ? meta[lane * 3 + 0] : 0x7fffffff;
-        int p = 0;
-        while (p < np) {
-            const int oy = __shfl_sync(0xffffffffu, my_oy, p);
-            // store the rows above oy: no later point reaches them
-            while (r0 < oy) flush_row();
-            const int q = 32 - __clz(__ballot_sync(0xffffffffu, my_oy == oy));
-            // float32: four points per unrolled step let the loads of the next points overlap the
-            // current FMAs; float64 keeps its registers for the accumulators
-            constexpr int UNR = F32 ? 4 : 1;
-#pragma unroll UNR
-            for (; p < q; ++p) {
-                // every lane loads (a column of the point's S x S block, clamped), and the
-                // lanes outside the block add zero: with no branch around the loads the
-                // unrolled points' coefficient loads are in flight together
-                const int sx = lane - meta[p * 3 + 1];
-                const bool act = sx >= 0 && sx < S;
-                const int sxc = min(max(sx, 0), S - 1);
-                const int i = meta[p * 3 + 2];
-                const cx<R> cv = act ? cst[p] : mk<R>(0, 0);
-                const cx<R>* cf = J.coef + (size_t)i * S * S + sxc;
+        const V* cf = reinterpret_cast<const V*>(J.coef + (size_t)(item.y + c0) * S * S);
+        constexpr int U = 4;
+        for (int p0 = 0; p0 < np; p0 += U) {
+            V b[U][NR];
 #pragma unroll
-                for (int k = 0; k < S; ++k) {
-                    const V2 b = __ldg(reinterpret_cast<const V2*>(cf + k * S));
-                    acc[k].x += b.x * cv.re + b.y * cv.im;   // conj(b) f
-                    acc[k].y += b.x * cv.im - b.y * cv.re;
+            for (int k = 0; k < U; ++k)
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    if (act[r] && p0 + k < np) b[k][r] = __ldg(cf + (size_t)(p0 + k) * NV + lane + 32 * r);
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                if (p0 + k >= np) break;   // uniform
+                const int op = __shfl_sync(0xffffffffu, o, p0 + k);
+                const R fr = __shfl_sync(0xffffffffu, f.re, p0 + k), fi = __shfl_sync(0xffffffffu, f.im, p0 + k);
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    if (!act[r]) continue;
+                    cx<R>* cell = pad + op + off[r];
+                    const R* bb = reinterpret_cast<const R*>(&b[k][r]);
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) {   // conj(b) f
+                        cell[v].re += bb[2 * v] * fr + bb[2 * v + 1] * fi;
+                        cell[v].im += bb[2 * v] * fi - bb[2 * v + 1] * fr;
+                    }
                 }
+                __syncwarp();
             }
         }
     }
-    // remaining rows (including rows no point reached)
-    while (r0 < P) flush_row();
+    __syncthreads();
+    const cx<R>* all = reinterpret_cast<const cx<R>*>(smem);
+    cx<R>* dst = J.padded + (size_t)it * cells;
+    for (int e = threadIdx.x; e < cells; e += 32 * NW) {
+        cx<R> v = all[e];
+#pragma unroll
+        for (int k = 1; k < NW; ++k) v = add(v, all[k * cells + e]);
+        dst[e] = v;
+    }
 }
 
-// warps per block: two of the tensor-core form, one of the float64 window form (its shared memory bounds the
-// warps per SM), four with B_opt
+// work items and warps per block: two of the tensor-core form, one of the float64 window form (its shared memory
+// bounds the warps per SM), one item on four warps with B_opt
 template <class R, bool BOPT>
-constexpr int spread2d_wpb() { return BOPT ? 4 : sizeof(R) == 4 ? 2 : 1; }
+constexpr int spread2d_wpb() { return !BOPT && sizeof(R) == 4 ? 2 : 1; }
+template <class R, bool BOPT>
+constexpr int spread2d_warps() { return BOPT ? SPREAD_BOPT_WARPS : spread2d_wpb<R, BOPT>(); }
 template <class R, int MM, bool BOPT>
 constexpr int spread2d_blocks() { return BOPT ? 1 : sizeof(R) == 4 ? (MM <= 4 ? 10 : 6) : 1; }
 
 template <class R, int MM, bool BOPT>
-__global__ void __launch_bounds__(32 * spread2d_wpb<R, BOPT>(), spread2d_blocks<R, MM, BOPT>())
+__global__ void __launch_bounds__(32 * spread2d_warps<R, BOPT>(), spread2d_blocks<R, MM, BOPT>())
     k_spread2d(const __grid_constant__ JobSet<R> js) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if constexpr (BOPT) {
+        spread2d_bopt_item<R, MM>(js, blockIdx.x, smem_raw);
+        return;
+    }
     const int warp = threadIdx.x >> 5;
     const int gitem = blockIdx.x * js.wpb + warp;
     if (gitem >= js.pre_items[js.njobs]) return;
     unsigned char* base = smem_raw + (size_t)warp * js.smem_per_warp;
-    if constexpr (BOPT) spread2d_bopt_item<R, MM>(js, gitem, base);
-    else if constexpr (sizeof(R) == 4) spread2d_mma_item<MM>(js, gitem, base);
+    if constexpr (BOPT) {
+    } else if constexpr (sizeof(R) == 4) spread2d_mma_item<MM>(js, gitem, base);
     else spread2d_f64_item<MM>(js, gitem, base);
 }
 
-// Per-launch setup: shared memory per warp (js.smem_per_warp), warps per block (js.wpb), and for
+// Per-launch setup: shared memory per item (js.smem_per_warp), items per block (js.wpb), and for
 // the tensor-core form the jobs' common window polynomial in the parameter block.
 template <class R, int MM, bool BOPT>
 static void spread2d_setup(JobSet<R>& js) {
     js.wpb = spread2d_wpb<R, BOPT>();
     js.wtab_ok = 0;
     if constexpr (BOPT) {
-        js.smem_per_warp = 32 * (int)sizeof(cx<R>) + 96 * (int)sizeof(int);
+        int P = 0;
+        for (int j = 0; j < js.njobs; ++j) P = std::max(P, js.job[j].P);
+        js.smem_per_warp = SPREAD_BOPT_WARPS * P * P * (int)sizeof(cx<R>);
     } else if constexpr (sizeof(R) == 4) {
         const size_t n = (size_t)WPOLY_ROWS * wpoly_stride(MM);
         bool same = js.job[0].wpoly_h != nullptr;
@@ -159,10 +161,10 @@ static infft_status launch_spread2d_m(JobSet<R>& js, cudaStream_t st) {
     if (nitems == 0) return INFFT_OK;
     const size_t smem = spw * js.wpb;
     INFFT_CUDA(cudaFuncSetAttribute(k_spread2d<R, MM, BOPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (!BOPT)   // shared memory bounds the warps per SM: ask for all of it
-        INFFT_CUDA(cudaFuncSetAttribute(k_spread2d<R, MM, BOPT>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                        (int)cudaSharedmemCarveoutMaxShared));
-    k_spread2d<R, MM, BOPT><<<(nitems + js.wpb - 1) / js.wpb, 32 * js.wpb, smem, st>>>(js);
+    // shared memory bounds the warps per SM: ask for all of it
+    INFFT_CUDA(cudaFuncSetAttribute(k_spread2d<R, MM, BOPT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    (int)cudaSharedmemCarveoutMaxShared));
+    k_spread2d<R, MM, BOPT><<<(nitems + js.wpb - 1) / js.wpb, 32 * spread2d_warps<R, BOPT>(), smem, st>>>(js);
     INFFT_LAUNCHED();
     return INFFT_OK;
 }
@@ -192,6 +194,7 @@ static bool spread2d_eligible(const JobSet<R>& js, int* m_out, bool* bopt_out) {
         // B_opt's extra slot): a tuned tile of 8 at m >= 5 (m >= 4 with B_opt) puts some cells
         // in three tiles along an axis, which the generic path handles
         if (J.P > 2 * J.T) return false;
+        if (bopt && ((uintptr_t)J.coef & 15)) return false;                 // 16-byte loads of coefficients
         if (sizeof(R) == 4 && !bopt && (J.P & 1)) return false;   // 16-byte stores of column pairs
     }
     if (m < 2 || m > 8) return false;   // m = 8 with window taps only: P = 16 + 16 <= 32
