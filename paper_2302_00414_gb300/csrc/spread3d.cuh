@@ -7,11 +7,13 @@
 #include <type_traits>
 
 #include "spread.cuh"
+#include "spreadmma3.cuh"
 
 namespace infft {
 
 // ---------------------------------------------------------------------------------------
-// Three-dimensional spreading (window modes), tiles of 8^3 cells.  One warp per work item,
+// Three-dimensional spreading (window modes), tiles of 8^3 cells, for float64 and for float32 with m = 5, 6 (smaller m:
+// spreadmma3.cuh).  One warp per work item,
 // the item's padded tile of P^3 cells (P = 8 + 2m, the window's taps) in shared memory.  Lane l takes
 // the (z, x) tap pairs q = l + 32 r of a point (W^2 pairs, ceil(W^2 / 32) rounds) and
 // holds the W cells of each pair along y in registers, adding (c_j psi_y) psi_z psi_x.
@@ -29,10 +31,9 @@ namespace infft {
 __host__ __device__ constexpr int spread3d_plane(int P, int W) { return P * P + (((W - P * P) % 16) + 16) % 16; }
 constexpr int SPREAD3D_T = 8;
 
-// points staged per chunk: 16 for float32 with m <= 4, so that a warp's tile and staging fit
-// six warps in an SM's shared memory (with 32 they fit five); 32 otherwise
+// points staged per chunk
 template <class R, int MM>
-__host__ __device__ constexpr int spread3d_chunk() { return (sizeof(R) == 4 && MM <= 4) ? 16 : 32; }
+__host__ __device__ constexpr int spread3d_chunk() { return 32; }
 
 // bytes of the per-warp prefetch slots (w, u triples, perm, cell of a chunk); a multiple of 16
 template <class R, int MM, bool PF>
@@ -246,16 +247,19 @@ static bool spread3d_eligible(const JobSet<R>& js, int* m_out) {
     return true;
 }
 
+// m = 1..4 in float32 take the tensor-core form (spread3d_try)
 template <class R, bool PF>
 static infft_status launch_spread3d(JobSet<R>& js, cudaStream_t st, int m) {
-    switch (m) {
-        case 1: return launch_spread3d_m<R, 1, PF>(js, st);
-        case 2: return launch_spread3d_m<R, 2, PF>(js, st);
-        case 3: return launch_spread3d_m<R, 3, PF>(js, st);
-        case 4: return launch_spread3d_m<R, 4, PF>(js, st);
-        case 5: return launch_spread3d_m<R, 5, PF>(js, st);
-        default: return launch_spread3d_m<R, 6, PF>(js, st);
+    if constexpr (sizeof(R) == 8) {
+        switch (m) {
+            case 1: return launch_spread3d_m<R, 1, PF>(js, st);
+            case 2: return launch_spread3d_m<R, 2, PF>(js, st);
+            case 3: return launch_spread3d_m<R, 3, PF>(js, st);
+            case 4: return launch_spread3d_m<R, 4, PF>(js, st);
+            default: break;
+        }
     }
+    return m == 5 ? launch_spread3d_m<R, 5, PF>(js, st) : launch_spread3d_m<R, 6, PF>(js, st);
 }
 
 static bool aligned3(const void* p, size_t a) { return ((uintptr_t)p & (a - 1)) == 0; }
@@ -281,6 +285,15 @@ infft_status spread3d_try(JobSet<R>& js, cudaStream_t st, bool* used) {
     *used = false;
     if (!spread3d_eligible(js, &m)) return INFFT_OK;
     *used = true;
+    if constexpr (sizeof(R) == 4) {   // tiles of 8^3: P = 8 + 2m is even and at most 16
+        switch (m) {
+            case 1: return launch_spread3d_mma<1>(js, st);
+            case 2: return launch_spread3d_mma<2>(js, st);
+            case 3: return launch_spread3d_mma<3>(js, st);
+            case 4: return launch_spread3d_mma<4>(js, st);
+            default: break;
+        }
+    }
     return spread3d_prefetch(js) ? launch_spread3d<R, true>(js, st, m) : launch_spread3d<R, false>(js, st, m);
 }
 
