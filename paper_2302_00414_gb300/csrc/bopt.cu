@@ -88,11 +88,13 @@ __global__ void k_bopt_sort(const int* __restrict__ start, long long ncols, long
 }
 
 // V(y) = sum_{k in I_M} w^(k) exp(2 pi i k y) for y = (u + m - s)/M_sigma, per point,
-// coordinate and slot.  exp(2 pi i k y) advances by rotation and is recomputed exactly
-// every 16 terms.
+// coordinate and slot.  w^ is even, so the terms k and -k make 2 w^(k) cos(2 pi k y) and only k = -M/2 stays
+// complex (half the terms and one product where two were taken).  exp(2 pi i k y) advances by rotation and
+// is recomputed exactly every 16 terms.
 __global__ void k_bopt_V(BoptGeom g, const double* __restrict__ x64, const double* __restrict__ what1,
                          cx<double>* __restrict__ V) {
     const long long total = (long long)g.N * g.d * g.S;
+    const int h = g.M / 2;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
         const int s = (int)(e % g.S);
         const long long it = e / g.S;  // i * d + t
@@ -100,29 +102,89 @@ __global__ void k_bopt_V(BoptGeom g, const double* __restrict__ x64, const doubl
         const double y = (u + (double)(g.m - s)) / (double)g.Ms;
         double sr, cr;
         sincospi(2.0 * y, &sr, &cr);  // one step
-        double acc_r = 0, acc_i = 0, zr = 0, zi = 0;
-        for (int k0 = 0; k0 < g.M; ++k0) {
-            if ((k0 & 15) == 0) sincospi(2.0 * y * (double)(k0 - g.M / 2), &zi, &zr);
-            const double wk = what1[k0];
-            acc_r += wk * zr;
-            acc_i += wk * zi;
+        double acc = 0, zr = 0, zi = 0;
+        for (int k = 1; k < h; ++k) {
+            if ((k & 15) == 1) sincospi(2.0 * y * (double)k, &zi, &zr);
+            acc += what1[h + k] * zr;
             const double nr = zr * cr - zi * sr, ni = zr * sr + zi * cr;
             zr = nr;
             zi = ni;
         }
-        V[e] = mk<double>(acc_r, acc_i);
+        double se, ce;
+        sincospi(-y * (double)g.M, &se, &ce);
+        V[e] = mk<double>(2.0 * acc + what1[h] + what1[0] * ce, what1[0] * se);
     }
 }
 
-// one factor of the Gram entries: D_{M/2-1}(u) + exp(-M pi i u), periodic in u
+// sin(pi r) and cos(pi r) for |r| <= 1/2 by their Taylor series (coefficients pi^k / k!, truncated below 2e-18 there):
+// within 2e-16 of the sine (relative) and of the cosine (absolute).  The Gram matrices take three of them per point pair
+// and axis; the library's functions, which reduce any argument, took twice the float64 instructions.
+__device__ __forceinline__ double sin_pi_half(double r) {
+    const double z = r * r;
+    double p = 5.392664662608129e-10;
+    p = fma(p, z, -2.2948428997269873e-08);
+    p = fma(p, z, 7.952054001475513e-07);
+    p = fma(p, z, -2.1915353447830217e-05);
+    p = fma(p, z, 0.00046630280576761255);
+    p = fma(p, z, -0.0073704309457143504);
+    p = fma(p, z, 0.08214588661112823);
+    p = fma(p, z, -0.5992645293207921);
+    p = fma(p, z, 2.5501640398773455);
+    p = fma(p, z, -5.16771278004997);
+    // pi = hi + lo
+    return fma(r, 3.141592653589793, r * fma(z, p, 1.2246467991473532e-16));
+}
+__device__ __forceinline__ double cos_pi_half(double r) {
+    const double z = r * r;
+    double p = -7.700707130601354e-11;
+    p = fma(p, z, 3.604730797462501e-09);
+    p = fma(p, z, -1.3878952462213771e-07);
+    p = fma(p, z, 4.303069587032947e-06);
+    p = fma(p, z, -0.0001046381049248457);
+    p = fma(p, z, 0.0019295743094039231);
+    p = fma(p, z, -0.02580689139001406);
+    p = fma(p, z, 0.2353306303588932);
+    p = fma(p, z, -1.3352627688545895);
+    p = fma(p, z, 4.0587121264167685);
+    p = fma(p, z, -4.934802200544679);
+    return fma(z, p, 1.0);
+}
+
+// sin and cos of pi u for |u| <= 1/8, where the series end earlier
+__device__ __forceinline__ void sincos_pi_eighth(double u, double& s, double& c) {
+    const double z = u * u;
+    double p = 0.00046630280576761255, q = -0.0001046381049248457;
+    q = fma(q, z, 0.0019295743094039231);
+    p = fma(p, z, -0.0073704309457143504);
+    q = fma(q, z, -0.02580689139001406);
+    p = fma(p, z, 0.08214588661112823);
+    q = fma(q, z, 0.2353306303588932);
+    p = fma(p, z, -0.5992645293207921);
+    q = fma(q, z, -1.3352627688545895);
+    p = fma(p, z, 2.5501640398773455);
+    q = fma(q, z, 4.0587121264167685);
+    p = fma(p, z, -5.16771278004997);
+    q = fma(q, z, -4.934802200544679);
+    s = fma(u, 3.141592653589793, u * fma(z, p, 1.2246467991473532e-16));
+    c = fma(z, q, 1.0);
+}
+
+// one factor of the Gram entries: D_{M/2-1}(u) + exp(-M pi i u), periodic in u; as sin(M pi u) (cot(pi u) - i)
+// it takes two sines, a cosine and a division (three sines, a cosine and a division before).  The members of a
+// column are 2m + 2 cells apart at most, so u is small on any but the smallest grids.
 __device__ __forceinline__ cx<double> gram_factor(double u, int M) {
     u -= rint(u);
-    double d;
-    if (u == 0.0) d = (double)(M - 1);
-    else d = sinpi((double)(M - 1) * u) / sinpi(u);
-    double s, c;
-    sincospi((double)M * u, &s, &c);
-    return mk<double>(d + c, -s);
+    if (u == 0.0) return mk<double>((double)M, 0.0);
+    const double v = (double)M * u, n = rint(v);
+    double sm = sin_pi_half(v - n), s, c;
+    if ((long long)n & 1) sm = -sm;
+    if (fabs(u) <= 0.125) {
+        sincos_pi_eighth(u, s, c);
+    } else {
+        s = sin_pi_half(u);
+        c = cos_pi_half(u);
+    }
+    return mk<double>(sm * c / s, -sm);
 }
 
 __host__ __device__ __forceinline__ long long tri(long long r, long long c) { return r * (r + 1) / 2 + c; }
@@ -136,8 +198,17 @@ __host__ __device__ __forceinline__ size_t bopt_fixed_bytes(int n, int d) {
 }
 
 // (row, column) of entry e of a packed lower triangle (e = r (r + 1) / 2 + c, c <= r): a
-// float estimate of the row, corrected by integer steps
+// float estimate of the row, corrected by integer steps (in 32 bits where the index allows)
 __device__ __forceinline__ void tri_rc(long long e, long long* r_out, long long* c_out) {
+    if (e < (1 << 30)) {
+        const int e32 = (int)e;
+        int r = (int)((sqrtf(8.f * (float)e32 + 1.f) - 1.f) * 0.5f);
+        while (r * (r + 1) / 2 > e32) --r;
+        while ((r + 1) * (r + 2) / 2 <= e32) ++r;
+        *r_out = r;
+        *c_out = e32 - r * (r + 1) / 2;
+        return;
+    }
     long long r = (long long)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
     while (r * (r + 1) / 2 > e) --r;
     while ((r + 1) * (r + 2) / 2 <= e) ++r;
@@ -172,7 +243,9 @@ __global__ void __launch_bounds__(BOPT_THREADS) k_bopt_solve(BoptGeom g, const i
     cx<double>* colk = yy + n_max;                                // n_max: current column of L
     double* xs = reinterpret_cast<double*>(colk + n_max);         // n_max * d
     long long* mem = reinterpret_cast<long long*>(xs + (size_t)n_max * g.d);  // n_max
-    __shared__ double s_diag;
+    // divisions cost some twenty instructions of the float64 pipe: one thread makes a pivot's reciprocal for all
+    // (made by every thread, in the factorisation and twice in the solves, they were half of the solver's time)
+    __shared__ double s_diag, s_inv;
     __shared__ int s_fail;
     __shared__ double s_trace;
     const int tid = threadIdx.x, nth = blockDim.x;
@@ -221,11 +294,14 @@ __global__ void __launch_bounds__(BOPT_THREADS) k_bopt_solve(BoptGeom g, const i
                 G[e] = v;
             }
             __syncthreads();
-            if (tid == 0) {
+            if (tid < 32) {
                 double tr = 0;
-                for (int j = 0; j < n; ++j) tr += G[tri(j, j)].re;
-                s_trace = tr;
-                s_fail = 0;
+                for (int j = tid; j < n; j += 32) tr += G[tri(j, j)].re;
+                for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+                if (tid == 0) {
+                    s_trace = tr;
+                    s_fail = 0;
+                }
             }
             __syncthreads();
             if (attempt > 0) {
@@ -239,11 +315,12 @@ __global__ void __launch_bounds__(BOPT_THREADS) k_bopt_solve(BoptGeom g, const i
                     const double dk = G[tri(k, k)].re;
                     if (!(dk > 0.0)) s_fail = 1;
                     s_diag = (dk > 0.0) ? sqrt(dk) : 1.0;
-                    G[tri(k, k)] = mk<double>(s_diag, 0.0);
+                    s_inv = 1.0 / s_diag;
+                    G[tri(k, k)] = mk<double>(s_diag, s_inv);   // the reciprocal beside it, for the solves
                 }
                 __syncthreads();
                 if (s_fail) break;
-                const double inv = 1.0 / s_diag;
+                const double inv = s_inv;
                 for (int i = k + 1 + tid; i < n; i += nth) {
                     const cx<double> l = scale(G[tri(i, k)], inv);
                     G[tri(i, k)] = l;
@@ -258,8 +335,9 @@ __global__ void __launch_bounds__(BOPT_THREADS) k_bopt_solve(BoptGeom g, const i
                     const int i = k + 1 + (int)ii, j = k + 1 + (int)jj;
                     const cx<double> li = colk[i], lj = colk[j];
                     cx<double> gij = G[tri(i, j)];
-                    gij.re -= li.re * lj.re + li.im * lj.im;  // l_i conj(l_j)
-                    gij.im -= li.im * lj.re - li.re * lj.im;
+                    // l_i conj(l_j), four multiply-adds (the float64 pipe binds this kernel)
+                    gij.re = fma(-li.re, lj.re, fma(-li.im, lj.im, gij.re));
+                    gij.im = fma(-li.im, lj.re, fma(li.re, lj.im, gij.im));
                     G[tri(i, j)] = gij;
                 }
                 __syncthreads();
@@ -276,28 +354,39 @@ __global__ void __launch_bounds__(BOPT_THREADS) k_bopt_solve(BoptGeom g, const i
         // L y = v (forward), L^* b = y (backward)
         for (int j = tid; j < n; j += nth) yy[j] = vv[j];
         __syncthreads();
+        // (a warp without rows left does no arithmetic)
+        const int first = tid & ~31;
         for (int c = 0; c < n; ++c) {
-            const double lcc = G[tri(c, c)].re;
-            const cx<double> yc = scale(yy[c], 1.0 / lcc);
+            const bool busy = c + 1 + first < n || first == 0;
+            cx<double> yc = mk<double>(0, 0);
+            if (busy) yc = scale(yy[c], G[tri(c, c)].im);
             __syncthreads();
             if (tid == 0) yy[c] = yc;
-            for (int r = c + 1 + tid; r < n; r += nth) yy[r] = sub(yy[r], mul(G[tri(r, c)], yc));
+            for (int r = c + 1 + tid; r < n; r += nth) {
+                const cx<double> l = G[tri(r, c)], y = yy[r];
+                yy[r] = mk<double>(fma(-l.re, yc.re, fma(l.im, yc.im, y.re)), fma(-l.re, yc.im, fma(-l.im, yc.re, y.im)));
+            }
             __syncthreads();
         }
         for (int c = n - 1; c >= 0; --c) {
-            const double lcc = G[tri(c, c)].re;
-            const cx<double> bc = scale(yy[c], 1.0 / lcc);
+            const bool busy = first < c || first == 0;
+            cx<double> bc = mk<double>(0, 0);
+            if (busy) bc = scale(yy[c], G[tri(c, c)].im);
             __syncthreads();
             if (tid == 0) yy[c] = bc;
-            for (int r = tid; r < c; r += nth) yy[r] = sub(yy[r], mulconj(G[tri(c, r)], bc));  // conj(L_cr) b_c
+            for (int r = tid; r < c; r += nth) {   // conj(L_cr) b_c
+                const cx<double> l = G[tri(c, r)], y = yy[r];
+                yy[r] = mk<double>(fma(-l.re, bc.re, fma(-l.im, bc.im, y.re)), fma(-l.re, bc.im, fma(l.im, bc.re, y.im)));
+            }
             __syncthreads();
         }
         // scatter b and the residual ||rhs||^2 - Re(b^* v)
         for (int j = tid; j < n; j += nth) coef[mem[j]] = yy[j];
-        if (tid == 0) {
+        if (tid < 32) {
             double re = 0;
-            for (int j = 0; j < n; ++j) re += yy[j].re * vv[j].re + yy[j].im * vv[j].im;
-            eps[col] = rhs2 - re;
+            for (int j = tid; j < n; j += 32) re += yy[j].re * vv[j].re + yy[j].im * vv[j].im;
+            for (int o = 16; o > 0; o >>= 1) re += __shfl_xor_sync(0xffffffffu, re, o);
+            if (tid == 0) eps[col] = rhs2 - re;
         }
         __syncthreads();
     }
@@ -438,44 +527,67 @@ static infft_status optimize_impl(infft_plan_s* p, unsigned opts, double* max_re
     long long n_smem = 0;
     while (n_smem < n_max && bopt_fixed_bytes((int)n_smem + 1, g.d) + (size_t)tri(n_smem + 2, 0) * 16 + 64 <= cap)
         ++n_smem;
-    std::vector<int> small, big;
-    int n_small = 0, n_big = 0;
+    // The shared-memory columns go out by size class, so that a block holds shared memory for a matrix of its
+    // class and not of the largest column, and has threads for its triangle: the factorisation is a chain
+    // of barriers and divisions that only other columns on the SM can fill (columns of 25 members:
+    // 18 blocks of 64 threads per SM where one class had 4 blocks of 256).
+    constexpr int CLASSES = 5;
+    const int bound[CLASSES] = {32, 48, 64, 96, 1 << 30}, threads[CLASSES] = {64, 64, 128, 128, BOPT_THREADS};
+    std::vector<int> small[CLASSES], big;
+    int n_cls[CLASSES] = {0}, n_big = 0;
+    size_t n_list = 0;
     for (long long c = 0; c < ncols; ++c) {
         const int n = hs[c + 1] - hs[c];
-        if (n <= n_smem) { small.push_back((int)c); n_small = std::max(n_small, n); }
-        else { big.push_back((int)c); n_big = std::max(n_big, n); }
+        if (n <= n_smem) {
+            int k = 0;
+            while (n > bound[k]) ++k;
+            small[k].push_back((int)c);
+            n_cls[k] = std::max(n_cls[k], n);
+        } else {
+            big.push_back((int)c);
+            n_big = std::max(n_big, n);
+        }
     }
+    for (const auto& v : small) n_list += v.size();
     std::stable_sort(big.begin(), big.end(), [&](int a, int b) { return hs[a + 1] - hs[a] > hs[b + 1] - hs[b]; });
     // The solve goes out in launches of about sixteen columns per block (tens of milliseconds
     // each), so that the blocks leave the SMs regularly and work of higher-priority streams (a
     // server's reconstructions while a new point set is admitted) is scheduled in between;
     // each launch has its own work counter.  (Two columns per block made the tails of the
     // launches cost half again the solve's time.)
-    int* list = (int*)alloc((small.size() + big.size()) * 4);
+    int* list = (int*)alloc((n_list + big.size()) * 4);
     if (!list) { set_error("optimize_B: out of device memory (column lists)"); return INFFT_ENOMEM; }
-    if (!small.empty())
-        INFFT_CUDA(cudaMemcpyAsync(list, small.data(), small.size() * 4, cudaMemcpyHostToDevice, st));
+    size_t pos = 0;
+    for (const auto& v : small) {
+        if (!v.empty()) INFFT_CUDA(cudaMemcpyAsync(list + pos, v.data(), v.size() * 4, cudaMemcpyHostToDevice, st));
+        pos += v.size();
+    }
     if (!big.empty())
-        INFFT_CUDA(cudaMemcpyAsync(list + small.size(), big.data(), big.size() * 4, cudaMemcpyHostToDevice, st));
-    if (!small.empty()) {
-        const size_t smem = bopt_fixed_bytes(std::max(n_small, 1), g.d) + (size_t)tri(n_small + 1, 0) * 16 + 64;
+        INFFT_CUDA(cudaMemcpyAsync(list + n_list, big.data(), big.size() * 4, cudaMemcpyHostToDevice, st));
+    pos = 0;
+    for (int k = 0; k < CLASSES; ++k) {
+        const std::vector<int>& v = small[k];
+        if (v.empty()) continue;
+        const int n_max = std::max(n_cls[k], 1);
+        const size_t smem = bopt_fixed_bytes(n_max, g.d) + (size_t)tri(n_cls[k] + 1, 0) * 16 + 64;
         int per_sm = 0;
         INFFT_CUDA(cudaFuncSetAttribute(k_bopt_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        INFFT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bopt_solve, BOPT_THREADS, smem));
+        INFFT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bopt_solve, threads[k], smem));
         const int blocks = nsm * std::max(1, per_sm);
         const long long chunk = 16LL * blocks;
-        const long long nchunk = ((long long)small.size() + chunk - 1) / chunk;
+        const long long nchunk = ((long long)v.size() + chunk - 1) / chunk;
         int* next = (int*)alloc((size_t)nchunk * 4);   // one work counter per launch
         if (!next) { set_error("optimize_B: out of device memory (work counters)"); return INFFT_ENOMEM; }
         INFFT_CUDA(cudaMemsetAsync(next, 0, (size_t)nchunk * 4, st));
         for (long long c = 0; c < nchunk; ++c) {
             const long long c0 = c * chunk;
-            const int n = (int)std::min<long long>(chunk, (long long)small.size() - c0);
-            k_bopt_solve<<<std::min(blocks, n), BOPT_THREADS, smem, st>>>(
-                g, start, members, p->x64, V, rhs2, list + c0, n, next + c, n_small, std::max(n_small, 1), nullptr, 1,
+            const int n = (int)std::min<long long>(chunk, (long long)v.size() - c0);
+            k_bopt_solve<<<std::min(blocks, n), threads[k], smem, st>>>(
+                g, start, members, p->x64, V, rhs2, list + pos + c0, n, next + c, n_cls[k], n_max, nullptr, 1,
                 nullptr, (cx<double>*)p->coef64, eps, status);
             INFFT_LAUNCHED();
         }
+        pos += v.size();
     }
     if (!big.empty()) {
         const bool fix_smem = bopt_fixed_bytes(n_big, g.d) + 64 <= cap;
@@ -505,7 +617,7 @@ static infft_status optimize_impl(infft_plan_s* p, unsigned opts, double* max_re
         for (size_t c = 0; c < nchunk; ++c) {
             const size_t c0 = c * (size_t)blocks;
             const int n = (int)std::min<size_t>((size_t)blocks, big.size() - c0);
-            k_bopt_solve<<<n, BOPT_THREADS, smem, st>>>(g, start, members, p->x64, V, rhs2, list + small.size() + c0, n,
+            k_bopt_solve<<<n, BOPT_THREADS, smem, st>>>(g, start, members, p->x64, V, rhs2, list + n_list + c0, n,
                                                          next + c, 0, n_big, gscr, fix_smem ? 1 : 0, gfix,
                                                          (cx<double>*)p->coef64, eps, status);
             INFFT_LAUNCHED();
