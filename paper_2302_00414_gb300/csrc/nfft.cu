@@ -182,8 +182,11 @@ __global__ void __launch_bounds__(256) k_merge2d(const __grid_constant__ JobSet<
 // Three-dimensional merge, one block per tile of T^3 cells (T a power of two, m < T),
 // threads striding over the tile's cells.  Along an axis the cell at offset r of tile t
 // lies in the padded tile of t at r + m, of t - 1 at r + T + m when that is < P, and of
-// t + 1 at r - T + m when that is >= 0; with T <= 2m both neighbours can hold it.  Work items of
-// a source tile are summed in item order, sources in a fixed order: deterministic.
+// t + 1 at r - T + m when that is >= 0.  With P <= 2 T at most one neighbour per axis holds it: the item ranges of
+// the 27 tiles around this one are read once per block, and the k-th items of a cell's (at most eight) sources are
+// loaded together before any is added (a range and a cell at a time, each waiting for the one before, took
+// 0.104 ms on the 128^3 grid of the spirals).  With T < 2m both neighbours can hold a cell.  Items and sources
+// are summed in a fixed order: deterministic.
 template <class R>
 __global__ void __launch_bounds__(256) k_merge3d(const __grid_constant__ JobSet<R> js) {
     const int gblk = blockIdx.x;
@@ -194,28 +197,67 @@ __global__ void __launch_bounds__(256) k_merge3d(const __grid_constant__ JobSet<
     const int tz = tile / (nt * nt), ty = (tile / nt) % nt, tx = tile % nt;
     const int logT = 31 - __clz(T);
     const size_t cells = (size_t)P * P * P;
+    __shared__ int s_i0[27], s_n[27];
+    if (threadIdx.x < 27) {
+        const int k = threadIdx.x, dz = k / 9 - 1, dy = k / 3 % 3 - 1, dx = k % 3 - 1;
+        const int tl = (((tz + dz + nt) % nt) * nt + (ty + dy + nt) % nt) * nt + (tx + dx + nt) % nt;
+        s_i0[k] = J.tile_items[tl];
+        s_n[k] = J.tile_items[tl + 1] - s_i0[k];
+    }
+    __syncthreads();
     for (int e = threadIdx.x; e < T * T * T; e += blockDim.x) {
-        const int rz = e >> (2 * logT), ry = (e >> logT) & (T - 1), rx = e & (T - 1);
-        const int rr[3] = {rz, ry, rx}, tt[3] = {tz, ty, tx};
-        int st[3][3], so[3][3], ns[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const int r = rr[a], t = tt[a];
-            st[a][0] = t; so[a][0] = r + m; ns[a] = 1;
-            if (r + T + m < P) { st[a][ns[a]] = (t - 1 + nt) % nt; so[a][ns[a]] = r + T + m; ++ns[a]; }
-            if (r - T + m >= 0) { st[a][ns[a]] = (t + 1) % nt; so[a][ns[a]] = r - T + m; ++ns[a]; }
-        }
+        const int rr[3] = {e >> (2 * logT), (e >> logT) & (T - 1), e & (T - 1)};
         cx<R> acc = mk<R>(0, 0);
-        for (int a = 0; a < ns[0]; ++a)
-            for (int b = 0; b < ns[1]; ++b)
-                for (int c = 0; c < ns[2]; ++c) {
-                    const int tl = (st[0][a] * nt + st[1][b]) * nt + st[2][c];
-                    const int i0 = __ldg(J.tile_items + tl), i1 = __ldg(J.tile_items + tl + 1);
-                    const size_t off = ((size_t)so[0][a] * P + so[1][b]) * P + so[2][c];
+        if (P <= 2 * T) {
+            int nb[3], so[3][2];   // the neighbour's position among the 27 (own: 1), offsets in own tile and neighbour
+            bool has[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int r = rr[a];
+                so[a][0] = r + m;
+                const bool lo = r + T + m < P, hi = r - T + m >= 0;
+                has[a] = lo || hi;
+                nb[a] = lo ? 0 : 2;
+                so[a][1] = lo ? r + T + m : r - T + m;
+            }
+            int cnt[8], top = 0;
+            size_t src[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int qz = q >> 2, qy = (q >> 1) & 1, qx = q & 1;
+                const bool ok = (!qz || has[0]) && (!qy || has[1]) && (!qx || has[2]);
+                const int k = ((qz ? nb[0] : 1) * 3 + (qy ? nb[1] : 1)) * 3 + (qx ? nb[2] : 1);
+                cnt[q] = ok ? s_n[k] : 0;
+                top = max(top, cnt[q]);
+                src[q] = (size_t)s_i0[k] * cells + ((size_t)so[0][qz] * P + so[1][qy]) * P + so[2][qx];
+            }
+#pragma unroll 1
+            for (int k = 0; k < top; ++k) {   // the k-th items of all sources together
+                cx<R> v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = k < cnt[q] ? J.padded[src[q] + (size_t)k * cells] : mk<R>(0, 0);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc = add(acc, v[q]);
+            }
+        } else {
+            int dt[3][3], so[3][3], ns[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int r = rr[a];
+                dt[a][0] = 1; so[a][0] = r + m; ns[a] = 1;
+                if (r + T + m < P) { dt[a][ns[a]] = 0; so[a][ns[a]] = r + T + m; ++ns[a]; }
+                if (r - T + m >= 0) { dt[a][ns[a]] = 2; so[a][ns[a]] = r - T + m; ++ns[a]; }
+            }
+            for (int a = 0; a < ns[0]; ++a)
+                for (int b = 0; b < ns[1]; ++b)
+                    for (int c = 0; c < ns[2]; ++c) {
+                        const int k = (dt[0][a] * 3 + dt[1][b]) * 3 + dt[2][c];
+                        const size_t off = ((size_t)so[0][a] * P + so[1][b]) * P + so[2][c];
 #pragma unroll 4
-                    for (int itm = i0; itm < i1; ++itm) acc = add(acc, J.padded[(size_t)itm * cells + off]);
-                }
-        J.grid[((size_t)(tz * T + rz) * Ms + ty * T + ry) * Ms + tx * T + rx] = acc;
+                        for (int itm = s_i0[k]; itm < s_i0[k] + s_n[k]; ++itm) acc = add(acc, J.padded[(size_t)itm * cells + off]);
+                    }
+        }
+        J.grid[((size_t)(tz * T + rr[0]) * Ms + ty * T + rr[1]) * Ms + tx * T + rr[2]] = acc;
     }
 }
 
