@@ -143,6 +143,55 @@ __device__ __forceinline__ void fft_stage(int L, int logL, int logn, int logNs, 
     }
 }
 
+// Sum of every padded-tile cell that maps onto grid cell `cidx` (row-major over Ms^D).
+template <class R, int D>
+__device__ __forceinline__ cx<R> merged_cell(const Job<R>& J, long long cidx) {
+    const int Ms = J.Ms, T = J.T, m = J.m, P = J.P, nt = J.ntile;
+    int c[D];
+    {
+        long long rem = cidx;
+        for (int t = D - 1; t >= 0; --t) { c[t] = (int)(rem % Ms); rem /= Ms; }
+    }
+    int cnt[D], tl[D][8], of[D][8];
+    for (int t = 0; t < D; ++t) {
+        cnt[t] = 0;
+        const int own = c[t] / T;
+        const int ncand = nt >= 3 ? 3 : nt;
+        for (int k = 0; k < ncand; ++k) {
+            const int tile = (nt >= 3) ? mod_pos(own - 1 + k, nt) : k;
+            int o = mod_pos(c[t] - tile * T + m, Ms);
+            for (; o < P && cnt[t] < 8; o += Ms) {
+                tl[t][cnt[t]] = tile;
+                of[t][cnt[t]] = o;
+                ++cnt[t];
+            }
+        }
+    }
+    const int cells = ipow(P, D);
+    cx<R> acc = mk<R>(0, 0);
+    int idx[D];
+    for (int t = 0; t < D; ++t) idx[t] = 0;
+    bool any = true;
+    for (int t = 0; t < D; ++t) any = any && cnt[t] > 0;
+    while (any) {
+        int tile_lin = 0, pidx = 0;
+        for (int t = 0; t < D; ++t) {
+            tile_lin = tile_lin * nt + tl[t][idx[t]];
+            pidx = pidx * P + of[t][idx[t]];
+        }
+        const int i0 = __ldg(J.tile_items + tile_lin), i1 = __ldg(J.tile_items + tile_lin + 1);
+        for (int itm = i0; itm < i1; ++itm) acc = add(acc, J.padded[(size_t)itm * cells + pidx]);
+        int t = D - 1;
+        while (t >= 0) {
+            if (++idx[t] < cnt[t]) break;
+            idx[t] = 0;
+            --t;
+        }
+        if (t < 0) break;
+    }
+    return acc;
+}
+
 // the sum of a cell over the items of its (at most four) sources, in order: item k of source q at
 // s_q + k cells.  Four loads in flight at a time (a dense centre's tile is split into dozens of items).
 template <class R>
@@ -167,7 +216,7 @@ __device__ __noinline__ cx<R> merge_items(const cx<R>* padded, unsigned cells, s
     return acc;
 }
 
-// With MRG (d = 2 adjoint, pass 0 only) the block's lines are grid rows whose cells are summed
+// With MRG (d = 1 and 2 adjoint, pass 0 only) the block's lines are grid rows whose cells are summed
 // from the padded tiles as they are loaded: the halo merge of k_merge2d in the same order per
 // cell, with no grid written or read in between.  The item ranges of the tiles the block's
 // rows draw on are staged in shared memory after the twiddles first.
@@ -201,7 +250,7 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
         if (sizeof(R) == 4) tws[skew(n >> 1) + 1 + skew(k)] = J.tw[(n >> 1) + k];
     }
     // then (merging pass only) the table of tile item ranges, then the M deconvolution factors
-    const int nrng = (MRG && pass == 0) ? mrg_tile_rows(L, J.T) * J.ntile : 0;
+    const int nrng = (MRG && D == 2 && pass == 0) ? mrg_tile_rows(L, J.T) * J.ntile : 0;
     int2* rng = reinterpret_cast<int2*>(tws + fft_tw_elems<R>(n));
     R* dvs = reinterpret_cast<R*>(rng + nrng);
     for (int k = threadIdx.x; k < (sizeof(R) == 4 ? 2 : 1) * M; k += NTH) dvs[k] = J.dinv[k];
@@ -241,7 +290,7 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
         s_out[tid] = bo;
     }
     int ty0 = 0, logT = 0, lognt = 0;
-    if (MRG && pass == 0) {
+    if (MRG && D == 2 && pass == 0) {
         const int T = J.T, nt = J.ntile;
         logT = 31 - __clz(T);
         lognt = 31 - __clz(nt);
@@ -258,7 +307,11 @@ __device__ __forceinline__ void fft_block(const JobSet<R>& js, const int pass, c
     // for n >= NTH (every line), else i = tid mod n on lines l = tid / n + (NTH / n) k.  The x-sources
     // of a column and the y-sources of a line are found once each; an element then looks up its (at most
     // four) tiles' item ranges.
-    if (MRG && pass == 0) {
+    if constexpr (MRG && D == 1) {   // one line, every cell from its own and the neighbouring tiles
+        for (int i = tid; i < L * n; i += NTH)
+            buf0[(i >> logn) * ns + skew(i & (n - 1))] = i < n ? merged_cell<R, 1>(J, i) : mk<R>(0, 0);
+        __syncthreads();
+    } else if (MRG && pass == 0) {
         const int T = J.T, m = J.m, P = J.P, nt = J.ntile;
         const unsigned cells = (unsigned)(P * P);
         const int ncol = n >= NTH ? n / NTH : 1, dl = n >= NTH ? 1 : NTH / n;
@@ -474,7 +527,7 @@ __device__ __forceinline__ void fft_conv_block(const JobSet<R>& js, const int lb
     }
 }
 
-// The halo merge of the d = 2 register-row path folded into the first FFT pass (fft_block with
+// The halo merge of d = 2 folded into the first FFT pass (fft_block with
 // MRG), unless INFFT_FFT_MERGE=0 or a job's table of tile item ranges would pass 16 KB: the
 // grid is then neither written nor read between the two.  Both forms give bitwise the same
 // result.

@@ -109,9 +109,6 @@ __global__ void __launch_bounds__(128) k_spread(const __grid_constant__ JobSet<R
     for (int e = lane; e < cells; e += 32) dst[e] = pad[e];
 }
 
-template <class R, int D>
-__device__ __forceinline__ cx<R> merged_cell(const Job<R>& J, long long cidx);
-
 // ---------------------------------------------------------------------------------------
 // Two-dimensional merge, one block per tile of T x T cells (T <= 16, T > m, Ms a multiple
 // of T), one thread per cell.  Along an axis, the cell at offset r in tile t lies in the
@@ -277,60 +274,11 @@ __global__ void __launch_bounds__(256) k_merge(const __grid_constant__ JobSet<R>
     J.grid[cidx] = merged_cell<R, D>(J, cidx);
 }
 
-// Sum of every padded-tile cell that maps onto grid cell `cidx` (row-major over Ms^D).
-template <class R, int D>
-__device__ __forceinline__ cx<R> merged_cell(const Job<R>& J, long long cidx) {
-    const int Ms = J.Ms, T = J.T, m = J.m, P = J.P, nt = J.ntile;
-    int c[D];
-    {
-        long long rem = cidx;
-        for (int t = D - 1; t >= 0; --t) { c[t] = (int)(rem % Ms); rem /= Ms; }
-    }
-    int cnt[D], tl[D][8], of[D][8];
-    for (int t = 0; t < D; ++t) {
-        cnt[t] = 0;
-        const int own = c[t] / T;
-        const int ncand = nt >= 3 ? 3 : nt;
-        for (int k = 0; k < ncand; ++k) {
-            const int tile = (nt >= 3) ? mod_pos(own - 1 + k, nt) : k;
-            int o = mod_pos(c[t] - tile * T + m, Ms);
-            for (; o < P && cnt[t] < 8; o += Ms) {
-                tl[t][cnt[t]] = tile;
-                of[t][cnt[t]] = o;
-                ++cnt[t];
-            }
-        }
-    }
-    const int cells = ipow(P, D);
-    cx<R> acc = mk<R>(0, 0);
-    int idx[D];
-    for (int t = 0; t < D; ++t) idx[t] = 0;
-    bool any = true;
-    for (int t = 0; t < D; ++t) any = any && cnt[t] > 0;
-    while (any) {
-        int tile_lin = 0, pidx = 0;
-        for (int t = 0; t < D; ++t) {
-            tile_lin = tile_lin * nt + tl[t][idx[t]];
-            pidx = pidx * P + of[t][idx[t]];
-        }
-        const int i0 = __ldg(J.tile_items + tile_lin), i1 = __ldg(J.tile_items + tile_lin + 1);
-        for (int itm = i0; itm < i1; ++itm) acc = add(acc, J.padded[(size_t)itm * cells + pidx]);
-        int t = D - 1;
-        while (t >= 0) {
-            if (++idx[t] < cnt[t]) break;
-            idx[t] = 0;
-            --t;
-        }
-        if (t < 0) break;
-    }
-    return acc;
-}
-
 // ---------------------------------------------------------------------------------------
 // float32: four 256-thread blocks per SM (64 registers hold a radix-8 butterfly), five of the merging pass,
 // whose loads want more threads (0.069 ms with four, 0.067 with five, 0.079 with six)
 template <class R, int D, bool FWD, bool MRG = false>
-__global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? (MRG ? 5 : 4) : 1)
+__global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? (MRG && D == 2 ? 5 : 4) : 1)
     k_fft(const __grid_constant__ JobSet<R> js, int pass) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fft_block<R, D, FWD, MRG, fft_threads<R>()>(js, pass, blockIdx.x, smem_raw);
@@ -587,6 +535,18 @@ static infft_status launch_adjoint(JobSet<R>& js, cudaStream_t st, cudaEvent_t* 
         INFFT_LAUNCHED();
     }
     if (ev) INFFT_CUDA(cudaEventRecord(ev[1], st));
+    if constexpr (D == 1) {
+        // the FFT pass sums the padded tiles as it loads (both forms give the same sums)
+        if (!grid_only && env_form("INFFT_FFT_MERGE") != 0) {
+            if (ev) INFFT_CUDA(cudaEventRecord(ev[2], st));
+            const size_t fsmem = fft_smem(js);
+            INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+            k_fft<R, 1, false, true><<<js.pre_fft[0][js.njobs], fft_threads<R>(), fsmem, st>>>(js, 0);
+            INFFT_LAUNCHED();
+            if (ev) INFFT_CUDA(cudaEventRecord(ev[3], st));
+            return INFFT_OK;
+        }
+    }
     k_merge<R, D><<<js.pre_merge[js.njobs], 256, 0, st>>>(js);
     INFFT_LAUNCHED();
     if (ev) INFFT_CUDA(cudaEventRecord(ev[2], st));
