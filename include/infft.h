@@ -128,14 +128,16 @@ infft_status infft_plan(int d, int M, int64_t N, const double* x, double sigma, 
  * has no counterpart; the values change speed only, never results beyond the rounding of
  * a different summation order (the spread tile and the item cap change which padded tiles
  * hold a point's taps, the others the schedule).  0 in a field keeps the library's default.
- *   tile      : edge T of the spreading tiles (a power of two, m < T <= M_sigma; the register-row
+ *   tile      : edge T of the spreading tiles (a power of two, m < T <= M_sigma; the fast
  *               spread of d = 2 needs T + 2m + 1 <= 32 and the fused merge-FFT kernel T in
  *               {8, 16}); default 16 for d = 2, 8 for d = 3, min(256, M_sigma) for d = 1.
- *   item_cap  : most points per work item, >= 1 (default 512; 32 for d = 1).
+ *   item_cap  : most points per work item, >= 1 (default 512; 128 for d = 2 in float64 up to
+ *               4 million points; 16 or 32 for d = 1).
  *   branches  : concurrent branches of batched adjoints with device buffers whose first plan
  *               is this one (1..8; default 3; batches with host buffers keep 8).
- *   prefetch  : spreading kernels copy the next points' data to shared memory while they
- *               spread the current ones: 1 on, 2 off (default: by form and grid size).
+ *   prefetch  : d = 3 spreading kernels of float64 and of m > 4 copy the next points' data to shared
+ *               memory while they spread the current ones: 1 on, 2 off (default on).
+ *               For d = 2, 2 keeps a batch off the persistent form, as INFFT_SPREAD2D_PREFETCH=0 does.
  *   fused_fft : d = 2 adjoints merge the padded tiles and run both FFT passes in one
  *               thread-block-cluster kernel: 1 on (where the grid fits), 2 off (default off).
  * An environment variable (INFFT_SPREAD2D_PREFETCH, INFFT_SPREAD3D_PREFETCH,
@@ -237,7 +239,7 @@ infft_status infft_get_bopt(infft_plan_t plan, void* coeff, void* stream);
  * spreads the current ones (those for d = 2 load them into registers and have no such choice).
  * INFFT_SPREAD3D_PREFETCH in the environment ("0" off, "1" on) overrides that choice; the
  * sums and their order, and so the results bit for bit, are the same either way.  So with
- * INFFT_FFT_MERGE (on unless "0"): for d = 2 the first FFT pass sums each grid cell from the
+ * INFFT_FFT_MERGE (on unless "0"): for d = 1 and d = 2 the first FFT pass sums each grid cell from the
  * padded tiles as it loads its rows (steps 2-3 of Algorithm 2.4 with no grid written in
  * between) instead of a separate halo-merge kernel.
  */

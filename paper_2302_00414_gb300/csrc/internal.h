@@ -31,6 +31,9 @@ struct infft_plan_s {
     double* x64 = nullptr;    // wrapped points in sorted order, N*d (B_opt, weights residual)
     int4* items = nullptr;
     int* tile_items = nullptr;
+    int4* items_long = nullptr;       // longer items, whose padded tiles fit infft_adjoint_noalloc's scratch where
+    int* tile_items_long = nullptr;   // those of `items` do not (nitems_long = 0: not needed)
+    int nitems_long = 0;
     int* cell_start = nullptr;  // key range + 1 prefix (tile-major cell order)
     size_t nkeys = 0;
 
@@ -93,6 +96,10 @@ void pool_free(void* ptr, cudaStream_t st);
 // waits for the stream's earlier work inside the driver and holds up the other host
 // threads' CUDA calls meanwhile; synchronising first leaves only the short copy.
 infft_status read_back(void* dst, const void* src, size_t bytes, cudaStream_t st);
+
+// infft_adjoint_noalloc's fixed scratch, and what a plan needs of it with `nitems` work items
+constexpr size_t INFFT_NOALLOC_SCRATCH_BYTES = 32u << 20;
+size_t noalloc_need(const infft_plan_s* p, long long nitems, size_t part[4]);
 
 // create a plan (argument checks of infft_plan); pooled plans use pool_alloc on `stream`
 infft_status plan_create(int d, int M, int64_t N, const double* x, double sigma, int m, unsigned flags,

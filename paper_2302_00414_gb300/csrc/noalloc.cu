@@ -11,11 +11,22 @@
 
 #include "internal.h"
 
-// 32 MiB of scratch per device, reserved for the lifetime of the process on every
-// device that loads the library.
-#define INFFT_NOALLOC_SCRATCH_BYTES (32ull << 20)
+// reserved on every device that loads the library, for the lifetime of the process
+static __device__ __align__(256) unsigned char g_noalloc_scratch[infft::INFFT_NOALLOC_SCRATCH_BYTES];
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[INFFT_NOALLOC_SCRATCH_BYTES];
+namespace infft {
+// bytes of the padded tiles, the grid and the FFT intermediates, each rounded to 256, and their sum
+size_t noalloc_need(const infft_plan_s* p, long long nitems, size_t part[4]) {
+    const size_t C = p->fp64 ? sizeof(cx<double>) : sizeof(cx<float>);
+    size_t tile = 1, grid = 1;
+    for (int t = 0; t < p->d; ++t) { tile *= (size_t)p->P; grid *= (size_t)p->Ms; }
+    const size_t cells[4] = {(size_t)std::max(1ll, nitems) * tile, grid, p->d >= 2 ? grid / p->Ms * p->M : 0,
+                             p->d == 3 ? (size_t)p->Ms * p->M * p->M : 0};
+    size_t need = 0;
+    for (int i = 0; i < 4; ++i) need += part[i] = (cells[i] * C + 255) & ~(size_t)255;
+    return need;
+}
+}  // namespace infft
 
 namespace {
 
@@ -87,35 +98,30 @@ infft_status scratch_address(void** out) {
     return INFFT_OK;
 }
 
-size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
-
 template <class R>
 infft_status run(infft_plan_s* p, int mode, const void* f, void* fhat, cudaStream_t st) {
     using infft::cx;
-    const int d = p->d;
-    size_t cells_p = 1, grid = 1;
-    for (int t = 0; t < d; ++t) { cells_p *= (size_t)p->P; grid *= (size_t)p->Ms; }
-    size_t t1 = 0, t2 = 0;
-    if (d >= 2) t1 = (size_t)infft::ipow(p->Ms, d - 1) * p->M;
-    if (d == 3) t2 = (size_t)p->Ms * p->M * p->M;
-    const size_t C = sizeof(cx<R>);
-    const size_t b_pad = round256(std::max<size_t>(1, (size_t)p->nitems) * cells_p * C);
-    const size_t b_grid = round256(grid * C);
-    const size_t b_t1 = round256(t1 * C), b_t2 = round256(t2 * C);
-    const size_t need = b_pad + b_grid + b_t1 + b_t2;
-    if (need > INFFT_NOALLOC_SCRATCH_BYTES) {
+    size_t part[4];
+    const bool longer = p->nitems_long > 0;  // the plan's shorter items do not fit
+    const size_t need = infft::noalloc_need(p, longer ? p->nitems_long : p->nitems, part);
+    if (need > infft::INFFT_NOALLOC_SCRATCH_BYTES) {
         infft::set_error("infft_adjoint_noalloc: plan needs %zu bytes of scratch, the fixed array holds %llu",
-                         need, (unsigned long long)INFFT_NOALLOC_SCRATCH_BYTES);
+                         need, (unsigned long long)infft::INFFT_NOALLOC_SCRATCH_BYTES);
         return INFFT_EINVAL;
     }
     void* base = nullptr;
     INFFT_TRY(scratch_address(&base));
     unsigned char* s = static_cast<unsigned char*>(base);
     infft::Job<R> job = infft::make_job<R>(p, mode, f, fhat);
+    if (longer) {
+        job.items = p->items_long;
+        job.tile_items = p->tile_items_long;
+        job.nitems = p->nitems_long;
+    }
     job.padded = reinterpret_cast<cx<R>*>(s);
-    job.grid = reinterpret_cast<cx<R>*>(s + b_pad);
-    job.tmp1 = t1 ? reinterpret_cast<cx<R>*>(s + b_pad + b_grid) : nullptr;
-    job.tmp2 = t2 ? reinterpret_cast<cx<R>*>(s + b_pad + b_grid + b_t1) : nullptr;
+    job.grid = reinterpret_cast<cx<R>*>(s + part[0]);
+    job.tmp1 = part[2] ? reinterpret_cast<cx<R>*>(s + part[0] + part[1]) : nullptr;
+    job.tmp2 = part[3] ? reinterpret_cast<cx<R>*>(s + part[0] + part[1] + part[2]) : nullptr;
     // Every scratch cell is written before it is read (the spread stores whole padded
     // tiles, the merge every grid cell where a separate merge runs, each FFT pass its whole
     // output; for d = 2 the first pass reads the padded tiles directly and the grid is not

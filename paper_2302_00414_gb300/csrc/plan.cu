@@ -444,9 +444,9 @@ template Job<double> make_job<double>(const infft_plan_s*, int, const void*, voi
 
 static void free_plan(infft_plan_s* p) {
     if (!p) return;
-    void* ptrs[] = {p->perm, p->cell, p->u, p->x64, p->items, p->tile_items, p->cell_start, p->dinv, p->tw,
-                    p->dinv_win, p->w_master, p->w_sorted, p->coef, p->coef64, p->padded, p->grid, p->tmp1,
-                    p->tmp2, p->io_in, p->io_out, p->wpoly};
+    void* ptrs[] = {p->perm, p->cell, p->u, p->x64, p->items, p->tile_items, p->items_long, p->tile_items_long,
+                    p->cell_start, p->dinv, p->tw, p->dinv_win, p->w_master, p->w_sorted, p->coef, p->coef64, p->padded,
+                    p->grid, p->tmp1, p->tmp2, p->io_in, p->io_out, p->wpoly};
     for (void* q : ptrs)
         if (q) { if (p->pooled) pool_free(q, p->pool_stream); else cudaFree(q); }
     for (const auto& e : p->extra)
@@ -553,25 +553,53 @@ static infft_status build_plan(infft_plan_s* p, const double* x_in, cudaStream_t
     std::vector<int> cs(nkeys + 1);
     INFFT_TRY(read_back(cs.data(), count, (size_t)(nkeys + 1) * 4, st));
     INFFT_CUDA(cudaStreamSynchronize(st));
-    // d = 1: short items so that a few hundred points still spread on several warps
-    const int cap = p->tune.item_cap > 0 ? p->tune.item_cap : (d == 1 ? 32 : 512);
+    // Points per work item.  d = 1: short items, so that a few hundred points spread on several warps (32 points,
+    // 16 where 32 would not give every SM one: 256 points 40.6 -> 32.8 us with the merge in the first FFT pass).
+    // d = 2 in float64: 128, since the spread takes a warp 1 us a point and a dense centre's items of 512 would leave
+    // a second wave of few warps (524,288 linogram points, m = 8: spread 1.395 -> 1.014 ms, first FFT pass 0.059 ->
+    // 0.133 ms); above 4 million points the waves are many and the padded tiles would grow by 100 bytes a point.
+    // Otherwise 512: the first FFT pass reads a padded tile per item (64-set float32 batch 299 -> 357 us with items
+    // of 96 points for the smaller sets).  Where the padded tiles of short items
+    // pass infft_adjoint_noalloc's scratch and those of long ones do not, the plan holds a list of long ones for it.
+    int nsm = 0, dev = 0;
+    INFFT_CUDA(cudaGetDevice(&dev));
+    INFFT_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int longest = d > 1 ? 512 : 32;
+    const int cap = p->tune.item_cap > 0 ? p->tune.item_cap
+                    : d == 2 && p->fp64 && N <= (4ll << 20) ? 128
+                    : d == 1 && N <= 32ll * nsm ? 16 : longest;
     std::vector<int4> items;
     std::vector<int> tile_items(ntiles + 1, 0);
-    for (int tl = 0; tl < ntiles; ++tl) {
-        tile_items[tl] = (int)items.size();
-        const int a = cs[(size_t)tl * tpow], b = cs[(size_t)(tl + 1) * tpow];
-        for (int s = a; s < b; s += cap) items.push_back(make_int4(tl, s, std::min(cap, b - s), 0));
-    }
-    tile_items[ntiles] = (int)items.size();
+    auto split = [&](int c) {
+        items.clear();
+        for (int tl = 0; tl < ntiles; ++tl) {
+            tile_items[tl] = (int)items.size();
+            const int a = cs[(size_t)tl * tpow], b = cs[(size_t)(tl + 1) * tpow];
+            for (int s = a; s < b; s += c) items.push_back(make_int4(tl, s, std::min(c, b - s), 0));
+        }
+        tile_items[ntiles] = (int)items.size();
+    };
+    auto to_device = [&](int4** di, int** dt) -> infft_status {
+        INFFT_TRY(dev_alloc(p, (void**)di, std::max<size_t>(1, items.size()) * sizeof(int4)));
+        INFFT_TRY(dev_alloc(p, (void**)dt, (size_t)(ntiles + 1) * 4));
+        if (!items.empty())
+            INFFT_CUDA(cudaMemcpyAsync(*di, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+        INFFT_CUDA(cudaMemcpyAsync(*dt, tile_items.data(), (size_t)(ntiles + 1) * 4, cudaMemcpyHostToDevice, st));
+        return INFFT_OK;
+    };
+    split(cap);
     p->nitems = (int)items.size();
-    INFFT_TRY(dev_alloc(p, (void**)&p->items, std::max<size_t>(1, items.size()) * sizeof(int4)));
-    INFFT_TRY(dev_alloc(p, (void**)&p->tile_items, (size_t)(ntiles + 1) * 4));
-    if (!items.empty())
-        INFFT_CUDA(cudaMemcpyAsync(p->items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-    INFFT_CUDA(cudaMemcpyAsync(p->tile_items, tile_items.data(), (size_t)(ntiles + 1) * 4, cudaMemcpyHostToDevice,
-                               st));
-
-
+    size_t part[4];
+    if (p->tune.item_cap == 0 && cap < longest && noalloc_need(p, p->nitems, part) > INFFT_NOALLOC_SCRATCH_BYTES) {
+        split(longest);
+        if (noalloc_need(p, (long long)items.size(), part) <= INFFT_NOALLOC_SCRATCH_BYTES) {
+            p->nitems_long = (int)items.size();
+            INFFT_TRY(to_device(&p->items_long, &p->tile_items_long));
+            INFFT_CUDA(cudaStreamSynchronize(st));  // the host vectors are filled anew
+        }
+        split(cap);
+    }
+    INFFT_TRY(to_device(&p->items, &p->tile_items));
 
     // tables
     INFFT_TRY(dev_alloc(p, &p->dinv, (size_t)p->M * (p->fp64 ? 1 : 2) * R_sz));
