@@ -243,9 +243,10 @@ __global__ void __launch_bounds__(BOPT_THREADS) k_bopt_solve(BoptGeom g, const i
     cx<double>* colk = yy + n_max;                                // n_max: current column of L
     double* xs = reinterpret_cast<double*>(colk + n_max);         // n_max * d
     long long* mem = reinterpret_cast<long long*>(xs + (size_t)n_max * g.d);  // n_max
-    // divisions cost some twenty instructions of the float64 pipe: one thread makes a pivot's reciprocal for all
-    // (made by every thread, in the factorisation and twice in the solves, they were half of the solver's time)
-    __shared__ double s_diag, s_inv;
+    // a root or a division costs some twenty instructions of the float64 pipe: one thread makes a pivot's reciprocal
+    // root for all (made by every thread, in the factorisation and twice in the solves, they were half of the
+    // solver's time)
+    __shared__ double s_inv;
     __shared__ int s_fail;
     __shared__ double s_trace;
     const int tid = threadIdx.x, nth = blockDim.x;
@@ -314,9 +315,8 @@ __global__ void __launch_bounds__(BOPT_THREADS) k_bopt_solve(BoptGeom g, const i
                 if (tid == 0) {
                     const double dk = G[tri(k, k)].re;
                     if (!(dk > 0.0)) s_fail = 1;
-                    s_diag = (dk > 0.0) ? sqrt(dk) : 1.0;
-                    s_inv = 1.0 / s_diag;
-                    G[tri(k, k)] = mk<double>(s_diag, s_inv);   // the reciprocal beside it, for the solves
+                    s_inv = (dk > 0.0) ? rsqrt(dk) : 1.0;
+                    G[tri(k, k)].im = s_inv;   // 1 / l_kk, for the solves (l_kk itself is not needed)
                 }
                 __syncthreads();
                 if (s_fail) break;
@@ -532,7 +532,7 @@ static infft_status optimize_impl(infft_plan_s* p, unsigned opts, double* max_re
     // of barriers and divisions that only other columns on the SM can fill (columns of 25 members:
     // 18 blocks of 64 threads per SM where one class had 4 blocks of 256).
     constexpr int CLASSES = 5;
-    const int bound[CLASSES] = {32, 48, 64, 96, 1 << 30}, threads[CLASSES] = {64, 64, 128, 128, BOPT_THREADS};
+    const int bound[CLASSES] = {32, 48, 64, 96, 1 << 30}, many[CLASSES] = {64, 64, 128, 128, BOPT_THREADS};
     std::vector<int> small[CLASSES], big;
     int n_cls[CLASSES] = {0}, n_big = 0;
     size_t n_list = 0;
@@ -570,9 +570,11 @@ static infft_status optimize_impl(infft_plan_s* p, unsigned opts, double* max_re
         if (v.empty()) continue;
         const int n_max = std::max(n_cls[k], 1);
         const size_t smem = bopt_fixed_bytes(n_max, g.d) + (size_t)tri(n_cls[k] + 1, 0) * 16 + 64;
+        // a few columns do not share an SM: all threads then, for the length of the one column's chain
+        const int nthr = (int)v.size() <= 2 * nsm ? BOPT_THREADS : many[k];
         int per_sm = 0;
         INFFT_CUDA(cudaFuncSetAttribute(k_bopt_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        INFFT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bopt_solve, threads[k], smem));
+        INFFT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bopt_solve, nthr, smem));
         const int blocks = nsm * std::max(1, per_sm);
         const long long chunk = 16LL * blocks;
         const long long nchunk = ((long long)v.size() + chunk - 1) / chunk;
@@ -582,7 +584,7 @@ static infft_status optimize_impl(infft_plan_s* p, unsigned opts, double* max_re
         for (long long c = 0; c < nchunk; ++c) {
             const long long c0 = c * chunk;
             const int n = (int)std::min<long long>(chunk, (long long)v.size() - c0);
-            k_bopt_solve<<<std::min(blocks, n), threads[k], smem, st>>>(
+            k_bopt_solve<<<std::min(blocks, n), nthr, smem, st>>>(
                 g, start, members, p->x64, V, rhs2, list + pos + c0, n, next + c, n_cls[k], n_max, nullptr, 1,
                 nullptr, (cx<double>*)p->coef64, eps, status);
             INFFT_LAUNCHED();
