@@ -239,7 +239,7 @@ infft_status infft_get_bopt(infft_plan_t plan, void* coeff, void* stream);
  * spreads the current ones (those for d = 2 load them into registers and have no such choice).
  * INFFT_SPREAD3D_PREFETCH in the environment ("0" off, "1" on) overrides that choice; the
  * sums and their order, and so the results bit for bit, are the same either way.  So with
- * INFFT_FFT_MERGE (on unless "0"): for d = 1 and d = 2 the first FFT pass sums each grid cell from the
+ * INFFT_FFT_MERGE (on unless "0"): for d = 2, and d = 1 on small grids, the first FFT pass sums each grid cell from the
  * padded tiles as it loads its rows (steps 2-3 of Algorithm 2.4 with no grid written in
  * between) instead of a separate halo-merge kernel.
  */

@@ -239,6 +239,7 @@ struct Job {
     const cx<R>* coef;         // B_opt coefficients, sorted order, N*S^d (BOPT)
     const int4* items;         // (tile, start, count, 0)
     const int* tile_items;     // ntile^d + 1 prefix of items per tile
+    const int* cell_start;     // sorted position of each cell's first point, cells tile-major
     const R* dinv;             // M entries 1/(Ms w^(k)) (per axis); float32: then their low parts
     const R* wpoly;            // wpoly_rows x wpoly_stride(m) window polynomial (Kaiser-Bessel plans) or null
     const float* wpoly_h;      // host copy of the same table (read by the launchers only) or null

@@ -179,7 +179,19 @@ __device__ __forceinline__ cx<R> merged_cell(const Job<R>& J, long long cidx) {
             tile_lin = tile_lin * nt + tl[t][idx[t]];
             pidx = pidx * P + of[t][idx[t]];
         }
-        const int i0 = __ldg(J.tile_items + tile_lin), i1 = __ldg(J.tile_items + tile_lin + 1);
+        int i0 = __ldg(J.tile_items + tile_lin), i1 = __ldg(J.tile_items + tile_lin + 1);
+        if (D == 1 && i1 - i0 > 1) {
+            // the points that touch padded cell o start at offsets o - S + 1 .. o of the tile: of its items, all of
+            // them as long as the first but the last, only those that hold such points (the others' cells are zeros).
+            // Float32, M_sigma = 128, 4,000 points: 35.4 us with all of them read (by a kernel of its own), 22.3 here.
+            const int S = J.mode == INFFT_MODE_BOPT ? J.S : 2 * m + 1;
+            const int a = __ldg(J.cell_start + tile_lin * T + max(0, pidx - S + 1));
+            const int b = __ldg(J.cell_start + tile_lin * T + min(T - 1, pidx) + 1);
+            const int4 first = __ldg(J.items + i0);
+            i1 = b > a ? i0 + (b - 1 - first.y) / first.z + 1 : i0;
+            i0 += (a - first.y) / first.z;
+        }
+#pragma unroll 4
         for (int itm = i0; itm < i1; ++itm) acc = add(acc, J.padded[(size_t)itm * cells + pidx]);
         int t = D - 1;
         while (t >= 0) {

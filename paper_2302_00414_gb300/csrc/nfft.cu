@@ -536,8 +536,13 @@ static infft_status launch_adjoint(JobSet<R>& js, cudaStream_t st, cudaEvent_t* 
     }
     if (ev) INFFT_CUDA(cudaEventRecord(ev[1], st));
     if constexpr (D == 1) {
-        // the FFT pass sums the padded tiles as it loads (both forms give the same sums)
-        if (!grid_only && env_form("INFFT_FFT_MERGE") != 0) {
+        // The FFT pass sums the padded tiles as it loads (both forms give the same sums), where its one block has at
+        // most two cells a thread; beyond that the merge wants a grid of blocks.  4 M points, merged on load against
+        // two kernels: float32 M_sigma = 128 / 512 / 2048 23.5 / 22.0 / 35.4 against 26.6 / 26.6 / 26.1 us, float64
+        // M_sigma = 128 / 512 / 2048 31.2 / 41.4 / 92.6 against 33.3 / 37.4 / 58.0 us.
+        bool on_load = !grid_only && env_form("INFFT_FFT_MERGE") != 0;
+        for (int j = 0; j < js.njobs; ++j) on_load = on_load && js.job[j].Ms <= 2 * fft_threads<R>();
+        if (on_load) {
             if (ev) INFFT_CUDA(cudaEventRecord(ev[2], st));
             const size_t fsmem = fft_smem(js);
             INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));

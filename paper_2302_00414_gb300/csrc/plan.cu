@@ -423,7 +423,7 @@ Job<R> make_job(const infft_plan_s* p, int mode, const void* in, void* out, int 
     J.beta = (R)p->beta; J.inv_m = (R)(1.0 / p->m);
     J.perm = p->perm; J.cell = p->cell; J.u = (const R*)p->u;
     J.w = (const cx<R>*)p->w_sorted; J.coef = (const cx<R>*)p->coef;
-    J.items = p->items; J.tile_items = p->tile_items;
+    J.items = p->items; J.tile_items = p->tile_items; J.cell_start = p->cell_start;
     J.dinv = (mode == INFFT_MODE_BOPT && p->dinv_win) ? (const R*)p->dinv_win : (const R*)p->dinv;
     J.tw = (const cx<R>*)p->tw;
     J.wpoly = (const R*)p->wpoly;

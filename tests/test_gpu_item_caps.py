@@ -39,3 +39,25 @@ def test_noalloc_accepts_plans_with_short_items(d, M, N, m, items):
             assert np.array_equal(a, b)
         else:
             assert rel(b, a) < 1e-13
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("M,N,m,points,tune", [
+    (64, 4000, 3, "random", None),            # one tile of 250 items
+    (1024, 5000, 8, "random", None),          # eight tiles, past the range of 16-point items
+    (64, 3001, 6, "cell", None),              # every point in two neighbouring cells, on a tile's edge
+    (8, 300, 5, "random", {"item_cap": 1}),   # a window wider than half of the grid, an item per point
+    (64, 2000, 4, "random", {"tile": 8, "item_cap": 3}),
+])
+def test_one_dimensional_merge_takes_the_items_of_a_cell(prec, tol, M, N, m, points, tune):
+    """The d = 1 merge visits only the items of a tile that hold points near the cell; against the oracle's
+    Algorithm 2.4 at the bounds of the other comparisons with it (float32: with exact sums of spreading)."""
+    from oracle import nfft as NF
+    L, torch = lib_or_skip()
+    x = inputs.random_points(N, 1, 9)
+    if points == "cell":
+        x = x * (2.0 / (2 * M))   # offsets -1 .. 1 of cells around 0, the edge of the first and the last tile
+    f = inputs.samples_complex(N, 10)
+    p = L.Plan(x, M, 2.0, m, prec, tune=tune)
+    h = p.adjoint(to_dev(torch, f, torch.complex64 if prec == "fp32" else torch.complex128), mode=L.MODE_PLAIN)
+    assert rel(h.cpu().numpy().ravel(), NF.adjoint_nfft(x, f, M, 2.0, m).ravel()) < tol
