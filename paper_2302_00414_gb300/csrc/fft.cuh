@@ -204,26 +204,30 @@ __device__ __forceinline__ cx<R> merged_cell(const Job<R>& J, long long cidx) {
     return acc;
 }
 
-// the sum of a cell over the items of its (at most four) sources, in order: item k of source q at
-// s_q + k cells.  Four loads in flight at a time (a dense centre's tile is split into dozens of items).
+// the sum of a cell over the items of its (at most four) sources, in order: item k of source q at s_q + k cells.
+// All sources' items are one sequence, U loads of it in flight: a polar centre's cell has dozens, and with four
+// at a time source by source its block's threads waited for one round of loads after the other (float32, 131,072 polar
+// points, m = 6, first FFT pass: 43 us so, 36 with eight of the sequence, 53 with sixteen; float64,
+// linogram of 524,288 points: 129 so, 142 with eight, 132 with sixteen; polar 112 with eight, 108 with sixteen).
 template <class R>
 __device__ __noinline__ cx<R> merge_items(const cx<R>* padded, unsigned cells, size_t s0, size_t s1, size_t s2, size_t s3,
                                           int n0, int n1, int n2, int n3) {
+    constexpr int U = sizeof(R) == 4 ? 8 : 16;
     cx<R> acc = mk<R>(0, 0);
+    const int p1 = n0, p2 = p1 + n1, p3 = p2 + n2, total = p3 + n3;
+    const cx<R>*b0 = padded + s0, *b1 = padded + s1, *b2 = padded + s2, *b3 = padded + s3;
 #pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-        const cx<R>* p = padded + (q == 0 ? s0 : q == 1 ? s1 : q == 2 ? s2 : s3);
-        const int n = q == 0 ? n0 : q == 1 ? n1 : q == 2 ? n2 : n3;
-        int k = 0;
-        for (; k + 4 <= n; k += 4) {
-            cx<R> v[4];
+    for (int k = 0; k < total; k += U) {
+        cx<R> v[U];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = p[(size_t)(k + i) * cells];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc = add(acc, v[i]);
+        for (int i = 0; i < U; ++i) {
+            const int e = k + i;
+            const cx<R>* b = e < p1 ? b0 : e < p2 ? b1 : e < p3 ? b2 : b3;
+            const unsigned f = (unsigned)(e - (e < p1 ? 0 : e < p2 ? p1 : e < p3 ? p2 : p3));
+            v[i] = e < total ? b[(size_t)f * cells] : mk<R>(0, 0);
         }
-#pragma unroll 1
-        for (; k < n; ++k) acc = add(acc, p[(size_t)k * cells]);
+#pragma unroll
+        for (int i = 0; i < U; ++i) acc = add(acc, v[i]);
     }
     return acc;
 }
