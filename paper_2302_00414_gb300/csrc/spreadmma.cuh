@@ -118,6 +118,7 @@ __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const
     if (use_poly && !js.wtab_ok)
         for (int e = lane; e < WPOLY_ROWS * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e] * wscale;
     for (int e = lane; e < C::OFF_META / 16; e += 32) reinterpret_cast<uint4*>(base)[e] = make_uint4(0, 0, 0, 0);
+    __syncwarp();   // before lanes read others' rows of the table and store taps over slots others cleared
 
     // acc[k][b]: row g of the k-th block of 8 rows held, columns 8b + 2t and 8b + 2t + 1; (x, y) real, (z, w)
     // imaginary parts (the two 8-row halves of an m16 tile)
