@@ -98,6 +98,12 @@ __host__ __device__ __forceinline__ float spread_mma_wscale(int wexp) {
 #endif
 }
 
+// The least exponent field e of a chunk's largest sample that is scaled up in full: the sum is scaled back by
+// 2^(e - 152 + w), w the window's exponent over all axes, which has to stay a power of two that float32 holds (2^-149; a
+// subnormal factor is exact).  Kaiser-Bessel windows (w >= 14) reach every normal sample, B-splines (w = 0) all but
+// the last two binades, where the products lie below float32's range in the first place.
+__device__ __forceinline__ int spread_mma_elow(int w) { return max(1, 3 - w); }
+
 // one warp spreads work item gitem (global over the JobSet's jobs); `base` is the warp's shared memory
 template <int MM>
 __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const int gitem, unsigned char* base) {
@@ -203,7 +209,7 @@ __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const
         load_point(c0);
         // 2^(126 - e) brings the chunk's samples to at most 1 (4 for the last exponents of float32)
         const unsigned top = __reduce_max_sync(0xffffffffu, lane < np ? __float_as_uint(fmaxf(fabsf(c.x), fabsf(c.y))) : 0u);
-        const int e = min(max((int)(top >> 23), 30), 252);
+        const int e = min(max((int)(top >> 23), spread_mma_elow(2 * J.wexp)), 252);
         const float cscale = __int_as_float((253 - e) << 23);
         const float us1 = __int_as_float((e + 1) << 23) * __int_as_float((127 + 2 * (J.wexp - 13)) << 23);
         const float us2 = us1 * 1.00000011920928955078125f;   // (1 + 2^-23): see above

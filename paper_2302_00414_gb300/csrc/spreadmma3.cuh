@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(64, 6) k_spread3d_mma(const __grid_constant__ 
         c0 += np;
         load_point(c0);
         const unsigned top = __reduce_max_sync(0xffffffffu, lane < mine ? __float_as_uint(fmaxf(fabsf(c.x), fabsf(c.y))) : 0u);
-        const int e = min(max((int)(top >> 23), 30), 252);
+        const int e = min(max((int)(top >> 23), spread_mma_elow(3 * J.wexp)), 252);
         const float cscale = __int_as_float((253 - e) << 23);
         if (lane < mine) {
             const int ra = C::OFF_A + (lane * C::SA + (lane >> 2)) * 8, rb = C::OFF_B + (lane * C::SB + (lane >> 2)) * 4;
