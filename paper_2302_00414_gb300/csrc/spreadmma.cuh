@@ -31,9 +31,10 @@ namespace infft {
 // of its maximum), the chunk's samples to at most 1, and the sum's scale is undone as it is added.  Each
 // group's sum starts from zero, the small part first, and is added to the accumulators by a float32
 // multiply-add: the tensor cores truncate their sums, which then costs at most one rounding of the
-// group's sum and not one of the running total.  The truncations shrink a group's sum by 3.7e-8 on
-// average (the grids' least-squares scale against float64: 1 - 3.7e-8 for random, polar and golden-angle
-// points alike); every other group is scaled up by 2^-23, which moves the mean to 1 + 2.3e-8.
+// group's sum and not one of the running total.  Truncation to 24 bits takes 2^-24 E[1 / mantissa], about 3.7e-8, off a
+// group's sum on average; the row factors are split with that much added (MMA_TRUNC), each point's alike, so that the mean
+// is kept whatever the number of points or groups.  (A factor of 1 + 2^-23 on every other group of a chunk kept it for full
+// chunks only, left sparse sets 3.5e-8 low and added its own 6e-8 of scatter to cells of one group.)
 //
 // A sample that is not finite makes NaN of its group's rows and columns of the tile (the form before:
 // of its 2m + 1 rows); after the transforms every coefficient is NaN either way.
@@ -66,12 +67,17 @@ struct SpreadMma {
     static_assert(W + 7 <= SA && W + 15 <= SB && 8 * RB <= SA && 8 * NB <= SB, "a window's taps and zeros");
 };
 
-// x c and y d as h + l in float16 (the product's own rounding goes into l): H and L hold (x's part, y's part)
+// x c and y d as h + l in float16 (the product's own rounding goes into l): H and L hold (x's part, y's part).  With
+// TRUNC both are larger by MMA_TRUNC, below the rounding of l and kept by it on average.
+constexpr float MMA_TRUNC = 3.7e-8f;
+template <bool TRUNC>
 __device__ __forceinline__ void split_f16(float x, float c, float y, float d, uint32_t& H, uint32_t& L) {
     const __half2 h = __floats2half2_rn(x * c, y * d);
     H = *reinterpret_cast<const uint32_t*>(&h);
     const float2 b = __half22float2(h);
-    const __half2 l = __floats2half2_rn(fmaf(x, c, -b.x), fmaf(y, d, -b.y));
+    float2 r = make_float2(fmaf(x, c, -b.x), fmaf(y, d, -b.y));
+    if (TRUNC) r = __ffma2_rn(b, make_float2(MMA_TRUNC, MMA_TRUNC), r);
+    const __half2 l = __floats2half2_rn(r.x, r.y);
     L = *reinterpret_cast<const uint32_t*>(&l);
 }
 
@@ -212,7 +218,7 @@ __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const
         const int e = min(max((int)(top >> 23), spread_mma_elow(2 * J.wexp)), 252);
         const float cscale = __int_as_float((253 - e) << 23);
         const float us1 = __int_as_float((e + 1) << 23) * __int_as_float((127 + 2 * (J.wexp - 13)) << 23);
-        const float us2 = us1 * 1.00000011920928955078125f;   // (1 + 2^-23): see above
+        const float2 us = make_float2(us1, us1);
         if (lane < np) {
             const int ra = C::OFF_A + (pos * C::SA + (pos >> 2)) * 8, rb = C::OFF_B + (pos * C::SB + (pos >> 2)) * 4;
             off = make_int2(ra - (oy & 7) * 8, rb - ox * 4);
@@ -222,14 +228,14 @@ __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const
 #pragma unroll
             for (int s = 0; s < W; ++s) {
                 uint32_t H, L;
-                split_f16(c.x, wt[0][s], c.y, wt[0][s], H, L);
+                split_f16<true>(c.x, wt[0][s], c.y, wt[0][s], H, L);
                 *reinterpret_cast<uint2*>(base + ra + 8 * s) =
                     make_uint2(__byte_perm(H, L, 0x5410), __byte_perm(H, L, 0x7632));
             }
 #pragma unroll
             for (int s = 0; s < W; s += 2) {
                 uint32_t H, L;
-                split_f16(wt[1][s], 1.f, s + 1 < W ? wt[1][s + 1] : 0.f, 1.f, H, L);
+                split_f16<false>(wt[1][s], 1.f, s + 1 < W ? wt[1][s + 1] : 0.f, 1.f, H, L);
                 *reinterpret_cast<uint32_t*>(base + rb + 4 * s) = __byte_perm(H, L, 0x5410);
                 if (s + 1 < W) *reinterpret_cast<uint32_t*>(base + rb + 4 * s + 4) = __byte_perm(H, L, 0x7632);
             }
@@ -259,7 +265,6 @@ __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const
                 const uint32_t v1 = *reinterpret_cast<const uint32_t*>(base + o1.y + 32 * b + 4 * g);
                 const uint32_t h0 = __byte_perm(v0, 0, 0x1010), l0 = __byte_perm(v0, 0, 0x3232);
                 const uint32_t h1 = __byte_perm(v1, 0, 0x1010), l1 = __byte_perm(v1, 0, 0x3232);
-                const float2 us = (grp & 1) ? make_float2(us2, us2) : make_float2(us1, us1);
                 float4 d[RB];
 #pragma unroll
                 for (int k = 0; k < RB; ++k)

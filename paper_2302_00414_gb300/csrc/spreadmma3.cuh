@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(64, 6) k_spread3d_mma(const __grid_constant__ 
                 for (int s = 0; s < W; ++s) {
                     if (a == 0) {
                         uint32_t H, L;
-                        split_f16(c.x, wt[0][s], c.y, wt[0][s], H, L);
+                        split_f16<true>(c.x, wt[0][s], c.y, wt[0][s], H, L);
                         *reinterpret_cast<uint2*>(own + ra + 8 * s) =
                             make_uint2(__byte_perm(H, L, 0x5410), __byte_perm(H, L, 0x7632));
                     } else if (a == 1) {
@@ -182,8 +182,7 @@ __global__ void __launch_bounds__(64, 6) k_spread3d_mma(const __grid_constant__ 
                 x1[b] = *reinterpret_cast<const float*>(half + o1.y + 32 * b + 4 * g);
             }
             if (grp == 0) load_sample(c0);
-            float us = *reinterpret_cast<const float*>(half + C::OFF_US);
-            if (grp & 1) us *= 1.00000011920928955078125f;   // (1 + 2^-23): centres the truncations, see spreadmma.cuh
+            const float us = *reinterpret_cast<const float*>(half + C::OFF_US);
             const float2 uu = make_float2(us, us);
             const float* pz0 = reinterpret_cast<const float*>(half + C::OFF_PZ) + p0 * W + s0;
             const float* pz1 = pz0 + 4 * W;
@@ -194,7 +193,7 @@ __global__ void __launch_bounds__(64, 6) k_spread3d_mma(const __grid_constant__ 
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
                     uint32_t H, L;
-                    split_f16(x0[b], w0, x1[b], w1, H, L);
+                    split_f16<false>(x0[b], w0, x1[b], w1, H, L);
                     const uint32_t h0 = __byte_perm(H, 0, 0x1010), h1 = __byte_perm(H, 0, 0x3232);
                     const uint32_t l0 = __byte_perm(L, 0, 0x1010), l1 = __byte_perm(L, 0, 0x3232);
                     float4 d[RB];
