@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "triangle.cuh"
 
 namespace infft {
 
@@ -187,33 +188,12 @@ __device__ __forceinline__ cx<double> gram_factor(double u, int M) {
     return mk<double>(sm * c / s, -sm);
 }
 
-__host__ __device__ __forceinline__ long long tri(long long r, long long c) { return r * (r + 1) / 2 + c; }
-
 constexpr int BOPT_THREADS = 256;
 
 // bytes of the per-column arrays (v, y, current column of L, member points, member ids),
 // rounded up to 256 so that consecutive per-block slices keep the 16-byte complex arrays aligned
 __host__ __device__ __forceinline__ size_t bopt_fixed_bytes(int n, int d) {
     return ((size_t)n * (16 * 3 + 8 * d + 8) + 255) & ~(size_t)255;
-}
-
-// (row, column) of entry e of a packed lower triangle (e = r (r + 1) / 2 + c, c <= r): a
-// float estimate of the row, corrected by integer steps (in 32 bits where the index allows)
-__device__ __forceinline__ void tri_rc(long long e, long long* r_out, long long* c_out) {
-    if (e < (1 << 30)) {
-        const int e32 = (int)e;
-        int r = (int)((sqrtf(8.f * (float)e32 + 1.f) - 1.f) * 0.5f);
-        while (r * (r + 1) / 2 > e32) --r;
-        while ((r + 1) * (r + 2) / 2 <= e32) ++r;
-        *r_out = r;
-        *c_out = e32 - r * (r + 1) / 2;
-        return;
-    }
-    long long r = (long long)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-    while (r * (r + 1) / 2 > e) --r;
-    while ((r + 1) * (r + 2) / 2 <= e) ++r;
-    *r_out = r;
-    *c_out = e - r * (r + 1) / 2;
 }
 
 // Persistent solver over a list of columns: each block takes the next column of `list`
