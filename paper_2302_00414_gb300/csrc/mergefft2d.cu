@@ -24,6 +24,7 @@
 #include "internal.h"
 #include "jobset.cuh"
 #include "spread.cuh"
+#include "fft.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -41,13 +42,14 @@ __device__ __forceinline__ int mf_skew(int i) { return i + (i >> 4); }
 // In-place decimation-in-time FFT (sign -) of nl lines of length n = 2^logn held in shared
 // memory in bit-reversed order: line l at buf + l * ls, element i at mf_skew(i).  Radix-4
 // steps (two radix-2 stages per thread in registers), one radix-2 stage first when logn is
-// odd.  tws: the n/2 twiddles exp(-2 pi i k / n).  Ends with a block barrier.
+// odd.  tws: the n/2 twiddles exp(-2 pi i k / n), in float32 followed by their low parts.  Ends with a block barrier.
 template <class R>
 __device__ void mf_fft_lines(cx<R>* buf, int nl, int ls, int n, int logn, const cx<R>* tws) {
     const int tid = threadIdx.x, nth = blockDim.x;
+    const int half_n = n >> 1;
     int lh = 0;
     if (logn & 1) {
-        const int half_n = n >> 1, loghn = logn - 1;
+        const int loghn = logn - 1;
         for (int e = tid; e < nl * half_n; e += nth) {
             const int l = e >> loghn, jj = e & (half_n - 1);
             cx<R>* row = buf + (size_t)l * ls;
@@ -68,17 +70,17 @@ __device__ void mf_fft_lines(cx<R>* buf, int nl, int ls, int n, int logn, const 
             cx<R>* row = buf + (size_t)l * ls;
             const cx<R> a0 = row[mf_skew(base)], a1 = row[mf_skew(base + q)];
             const cx<R> a2 = row[mf_skew(base + 2 * q)], a3 = row[mf_skew(base + 3 * q)];
-            const cx<R> w1 = tws[pos << (logn - 1 - lh)];
-            const cx<R> w2 = tws[pos << (logn - 2 - lh)];
-            const cx<R> w3 = tws[(pos + q) << (logn - 2 - lh)];
-            cx<R> t = mul(w1, a1);
+            const int i1 = pos << (logn - 1 - lh), i2 = pos << (logn - 2 - lh), i3 = (pos + q) << (logn - 2 - lh);
+            auto low = [&](int i) { return sizeof(R) == 4 ? tws[half_n + i] : mk<R>(0, 0); };
+            const cx<R> w1 = tws[i1], w1l = low(i1);
+            cx<R> t = mul_w(a1, w1, w1l);
             const cx<R> b0 = add(a0, t), b1 = sub(a0, t);
-            t = mul(w1, a3);
+            t = mul_w(a3, w1, w1l);
             const cx<R> b2 = add(a2, t), b3 = sub(a2, t);
-            t = mul(w2, b2);
+            t = mul_w(b2, tws[i2], low(i2));
             row[mf_skew(base)] = add(b0, t);
             row[mf_skew(base + 2 * q)] = sub(b0, t);
-            t = mul(w3, b3);
+            t = mul_w(b3, tws[i3], low(i3));
             row[mf_skew(base + q)] = add(b1, t);
             row[mf_skew(base + 3 * q)] = sub(b1, t);
         }
@@ -89,7 +91,7 @@ __device__ void mf_fft_lines(cx<R>* buf, int nl, int ls, int n, int logn, const 
 // shared-memory layout of one CTA (sizes in elements)
 struct MfLayout {
     int RB, ns, CW, cs;          // rows per CTA, row stride, columns per CTA, column stride
-    size_t rc, cmp, tw;          // row / column region, compact rows, twiddles (complex)
+    size_t rc, cmp, tw;          // row / column region, compact rows, twiddles and (float32) their low parts (complex)
     int NR;                      // contributing tile rows
     size_t bytes;
 };
@@ -104,9 +106,9 @@ __host__ __device__ inline MfLayout mf_layout(int Ms, int M, int nt, int T, int 
     const size_t rows = (size_t)L.RB * L.ns, cols = (size_t)L.CW * L.cs;
     L.rc = rows > cols ? rows : cols;
     L.cmp = (size_t)L.RB * M;
-    L.tw = (size_t)(Ms / 2);
+    L.tw = (size_t)(Ms / 2) * (sizeof(R) == 4 ? 2 : 1);
     L.NR = CS == 1 ? nt : L.RB / T + 2;
-    L.bytes = (L.rc + L.cmp + L.tw) * sizeof(cx<R>) + (size_t)M * sizeof(R) + (size_t)L.NR * (nt + 1) * sizeof(int) +
+    L.bytes = (L.rc + L.cmp + L.tw) * sizeof(cx<R>) + (size_t)M * fft_dv_bytes<R>() + (size_t)L.NR * (nt + 1) * sizeof(int) +
               64;
     return L;
 }
@@ -124,14 +126,16 @@ __global__ void __launch_bounds__(MF_THREADS, 1) k_mergefft2d(const __grid_const
     const int y0 = rank * RB, c0 = rank * CW;
     cx<R>* rc = reinterpret_cast<cx<R>*>(smem_raw);       // rows RB x ns, later columns CW x cs
     cx<R>* cmp = rc + Lo.rc;                               // compact rows RB x M
-    cx<R>* tws = cmp + Lo.cmp;                             // Ms/2 twiddles
-    R* dv = reinterpret_cast<R*>(tws + Lo.tw);             // M deconvolution factors
-    int* titem = reinterpret_cast<int*>(dv + M);           // NR x (nt + 1) item prefix per tile row
+    cx<R>* tws = cmp + Lo.cmp;                             // Ms/2 twiddles, in float32 their low parts
+    constexpr int DV = sizeof(R) == 4 ? 2 : 1;
+    R* dv = reinterpret_cast<R*>(tws + Lo.tw);             // M deconvolution factors, in float32 their low parts
+    int* titem = reinterpret_cast<int*>(dv + DV * M);      // NR x (nt + 1) item prefix per tile row
     const int tid = threadIdx.x, nth = blockDim.x;
     const int ty_first = CS == 1 ? 0 : y0 / T - 1;        // unwrapped tile row of contributing row 0
 
-    for (int k = tid; k < (Ms >> 1); k += nth) tws[k] = J.tw[k];
-    for (int k = tid; k < M; k += nth) dv[k] = J.dinv[k];
+    for (int k = tid; k < (int)Lo.tw; k += nth) tws[k] = J.tw[k];
+    for (int k = tid; k < DV * M; k += nth) dv[k] = J.dinv[k];
+    auto low = [&](int k) { return DV == 2 ? dv[M + k] : R(0); };
     for (int e = tid; e < NR * (nt + 1); e += nth) {
         const int r = e / (nt + 1), tx = e - r * (nt + 1);
         const int ty = mod_pos(ty_first + r, nt);
@@ -213,7 +217,7 @@ __global__ void __launch_bounds__(MF_THREADS, 1) k_mergefft2d(const __grid_const
     mf_fft_lines<R>(rc, RB, ns, Ms, logn, tws);
     for (int e = tid; e < RB * M; e += nth) {
         const int yl = e / M, i = e - yl * M;
-        cmp[e] = scale(rc[yl * ns + mf_skew(mod_pos(i - M / 2, Ms))], dv[i]);
+        cmp[e] = mul_d(rc[yl * ns + mf_skew(mod_pos(i - M / 2, Ms))], dv[i], low(i));
     }
 
     // 3. gather this CTA's columns from every CTA of the cluster, column FFTs, crop, deconvolve
@@ -237,7 +241,7 @@ __global__ void __launch_bounds__(MF_THREADS, 1) k_mergefft2d(const __grid_const
     mf_fft_lines<R>(rc, CW, cs, Ms, logn, tws);
     for (int e = tid; e < M * CW; e += nth) {
         const int k0 = e / CW, kk = e - k0 * CW;
-        J.out[(size_t)k0 * M + c0 + kk] = scale(rc[kk * cs + mf_skew(mod_pos(k0 - M / 2, Ms))], dv[k0]);
+        J.out[(size_t)k0 * M + c0 + kk] = mul_d(rc[kk * cs + mf_skew(mod_pos(k0 - M / 2, Ms))], dv[k0], low(k0));
     }
 }
 
