@@ -352,8 +352,12 @@ infft_status mergefft2d_try(const JobSet<R>& js, cudaStream_t st, std::vector<in
         JobSel sel;
         sel.n = (int)g.second.size();
         for (int i = 0; i < sel.n; ++i) sel.job[i] = g.second[i];
-        const Job<R>& J0 = js.job[g.second[0]];
-        const size_t smem = mf_layout<R>(J0.Ms, J0.M, J0.ntile, J0.T, CS).bytes;
+        // a group's jobs may differ in M (other oversampling of one grid size), and with it in their layout
+        size_t smem = 0;
+        for (int j : g.second) {
+            const Job<R>& J = js.job[j];
+            smem = std::max(smem, mf_layout<R>(J.Ms, J.M, J.ntile, J.T, CS).bytes);
+        }
         bool ok = false;
         switch (CS) {
             case 1: status = mf_launch<R, 1>(js, sel, smem, gs, &ok); break;

@@ -37,3 +37,21 @@ def test_gain_of_the_bins(M, form, monkeypatch):
     gain = (num / den).cpu().numpy()
     assert np.isfinite(gain).all()
     assert math.sqrt(((gain - gain.mean()) ** 2).mean()) < U / 3
+
+
+@pytest.mark.parametrize("order", [(24, 32, 28), (32, 24, 28)])
+def test_fused_batch_of_degrees_on_one_grid(order, monkeypatch):
+    """Jobs of one grid size and different degrees share a launch of the fused kernel: each has the shared memory of
+    the largest layout, and the result of its own call bit for bit."""
+    L, torch = lib_or_skip()
+    monkeypatch.setenv("INFFT_FUSED_MERGE_FFT", "1")
+    plans, fs, hs, alone = [], [], [], []
+    for i, M in enumerate(order):
+        plans.append(L.Plan(inputs.random_points(900 + i, 2, 92 + i), M, 63.5 / M, 4, "fp32"))
+        fs.append(torch.from_numpy(inputs.samples_complex(900 + i, 95 + i)).to("cuda", torch.complex64))
+        hs.append(torch.empty((M, M), dtype=torch.complex64, device="cuda"))
+        alone.append(plans[-1].adjoint(fs[-1]).cpu().numpy())
+    assert {p.Ms for p in plans} == {64}
+    L.adjoint_batched(plans, fs, hs, L.MODE_PLAIN)
+    for h, a in zip(hs, alone):
+        assert np.array_equal(h.cpu().numpy(), a)
