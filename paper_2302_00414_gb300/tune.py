@@ -4,10 +4,11 @@ For a workload -- a list of point sets of one dimension, precision and window wi
 are reconstructed together as one batched, graph-replayed adjoint -- the tuner times the
 batch under candidate choices and keeps the fastest:
 
-  tile       spreading tile edge T (d = 2: 16 or 8; the register-row spread needs
+  tile       spreading tile edge T (d = 2: 16 or 8; the fixed-m spreads need
              T + 2m + 1 <= 32, so larger tiles are not candidates)
   item_cap   most points per work item (256, 512, 1024)
-  prefetch   the spreads' copy of the next points' data to shared memory (on / off)
+  prefetch   d = 3: the spreads' copy of the next points' data to shared memory (on / off); the spreads
+             of d = 2 have no such choice
   fused_fft  the d = 2 cluster kernel that fuses the halo merge with both FFT passes
   branches   concurrent branches of the batch (1, 2, 3, 4, 6)
 
@@ -32,8 +33,7 @@ from . import api as A
 HERE = os.path.dirname(os.path.abspath(__file__))
 DEFAULT_CACHE = os.path.join(HERE, "tuning.json")
 
-CANDIDATES_2D = {"item_cap": [256, 512, 1024], "prefetch": [1, 2], "fused_fft": [1, 2],
-                 "branches": [1, 2, 3, 4, 6], "tile": [16, 8]}
+CANDIDATES_2D = {"item_cap": [256, 512, 1024], "fused_fft": [1, 2], "branches": [1, 2, 3, 4, 6], "tile": [16, 8]}
 CANDIDATES_3D = {"item_cap": [256, 512, 1024], "prefetch": [1, 2], "branches": [1, 2, 3, 4, 6]}
 
 
@@ -152,6 +152,9 @@ def tuned_choice(L, torch, sets, fs, m: int = 4, precision: str = "fp32", mode: 
     cache = load_cache(cache_path)
     if key in cache and not retune:
         out = dict(cache[key])
+        # a choice the dimension no longer has (prefetch for d = 2, where 2 would only keep a batch off the persistent form)
+        fields = CANDIDATES_2D if sets[0][1].shape[1] == 2 else CANDIDATES_3D
+        out["tune"] = {k: v for k, v in out["tune"].items() if k in fields}
         out["source"] = "cache"
         out["key"] = key
         return out
