@@ -27,6 +27,7 @@ from __future__ import annotations
 
 import collections
 import dataclasses
+import math
 import queue
 import threading
 import time
@@ -55,6 +56,20 @@ class PointSet:
     x: Any                   # N x d float64 (host), or a callable returning it
     precision: str = "fp32"
     N: int = 0               # number of points (needed when x is a callable)
+
+
+def plan_size(n: int, d: int, M: int, Ms: int, m: int, fp64: bool) -> int:
+    """Device bytes of a plan with the library's default tiles: sorted points, work items with their padded tiles (a tile's
+    last item may be short, so at most one more than n over the item's points for each tile that holds points),
+    grid, FFT intermediates and the cells' prefix.  Short items make the padded tiles the largest part: 128 points of
+    d = 2 in float64 share a tile of 25 x 25 (m = 4) to 33 x 33 cells (m = 8)."""
+    C = 16 if fp64 else 8
+    T = min({1: 256, 2: 16, 3: 8}[d], Ms)
+    cap = 16 if d == 1 else 128 if d == 2 and fp64 and n <= 4 << 20 else 512
+    items = min(n, (-(-Ms // T)) ** d) + n // cap
+    grid = Ms ** d
+    tmp = (Ms ** (d - 1) * M if d >= 2 else 0) + (Ms * Ms * M if d == 3 else 0)
+    return n * (8 + d * (C // 2 + 8)) + items * ((T + 2 * m + 1) ** d * C + 32) + (grid + tmp) * C + 8 * grid + 64 * Ms
 
 
 class Backend:
@@ -99,13 +114,22 @@ class Backend:
         return plan.device_bytes
 
     def estimate_bytes(self, ps: PointSet) -> int:
+        """Device memory that building and keeping a point set takes at its peak: the plan with its weights, and beside
+        it the degree-2M float64 plan, vectors and convolution buffers of the weights' CG."""
         n = ps.N if ps.N else ps.x.shape[0]
-        grid = (2 * ps.M) ** ps.d
-        cg = 16 * ((4 * ps.M) ** ps.d) * 8   # float64 grids and scratch of the degree-2M solve
+        d, M = ps.d, ps.M
+        fp64 = ps.precision == "fp64"
+        own = plan_size(n, d, M, 2 * math.ceil(math.ceil(self.sigma * M) / 2), self.m, fp64) + n * (16 + (16 if fp64 else 8))
+        K, L = (2 * M) ** d, (4 * M) ** d
+        cg = 16 * (5 * max(n, K) + max(n, K) + n + K)
+        if K <= n and 4 * M <= 4096:     # the Toeplitz form: its spectrum, grid and FFT intermediates, modulated samples
+            cg += 16 * ((d + 1) * L + n + K)
+        sub = plan_size(n, d, 2 * M, 4 * M, 8 if d <= 2 else 4, True)
+        build = n * (24 * d + 12) + 4 * L   # sorting a plan's points
         extra = 0
-        if self.bopt and ps.d == 2:   # float64 and plan-precision coefficients, member lists and V
-            extra = n * (2 * self.m + 2) ** ps.d * (16 + 8 + 8) + 16 * n * ps.d * (2 * self.m + 2)
-        return 120 * n + 40 * grid + cg + extra
+        if self.bopt and d == 2:   # float64 and plan-precision coefficients, member lists and V
+            extra = n * (2 * self.m + 2) ** d * (16 + 8 + 8) + 16 * n * d * (2 * self.m + 2)
+        return own + max(build, sub + max(build, cg), extra)
 
     def free_bytes(self) -> int:
         # the device query can wait behind another thread's synchronising call (a plan's
