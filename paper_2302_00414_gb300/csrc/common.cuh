@@ -163,8 +163,9 @@ __device__ __forceinline__ void poly_taps(const float* __restrict__ c, const flo
 }
 
 // Float64 plans: the same polynomials of degree 21 (from values to twice the precision, made on the host at
-// plan creation), which reach the rounding level of float64 for any oversampling: the window over one cell
-// varies no faster than exp(pi v), whose Chebyshev coefficients fall below 2e-17 there.  A tap costs 11
+// plan creation: polytable.h).  Interpolation is off by at most 1e-23 of the window's largest value for every m and
+// oversampling, and by less than 1e-17 of a tap's own largest value but for the outermost taps of m > 10 with
+// M < M_sigma / 2 (5e-14 for m = 15, M = M_sigma / 10, where that tap is 2e-25 of the window).  A tap costs 11
 // multiply-adds; the double Bessel function cost several times that, at 1/32 of the float32 rate.
 constexpr int WPOLY64_DEG = 21;
 constexpr int WPOLY64_ROWS = WPOLY64_DEG + 1;

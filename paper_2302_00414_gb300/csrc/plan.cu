@@ -11,6 +11,7 @@
 
 #include "internal.h"
 #include "jobset.cuh"
+#include "polytable.h"
 
 namespace infft {
 
@@ -336,61 +337,8 @@ __global__ void k_wpoly(int m, double beta, float* __restrict__ coef) {
     coef[P1 * WP + i] = (float)(a[0] - (double)(float)a[0]);
 }
 
-// Window polynomials for float64 Kaiser-Bessel plans, on the host in double-double arithmetic (Dekker / Knuth
-// error-free sums and products): tap s = 1..m is interpolated at the 22 Chebyshev points of v in Newton's form,
-// phi from the power series of I0, and rewritten in powers of v.  The last tables are kept (a program's plans, and
-// the weights' inner plans, share a few windows).
-namespace {
-struct dd { double h, l; };
-dd two_sum(double a, double b) { const double s = a + b, t = s - a; return {s, (a - (s - t)) + (b - t)}; }
-dd operator+(dd a, dd b) { dd s = two_sum(a.h, b.h); s.l += a.l + b.l; return two_sum(s.h, s.l); }
-dd operator-(dd a) { return {-a.h, -a.l}; }
-dd operator*(dd a, dd b) {
-    const double p = a.h * b.h, e = std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h);
-    return two_sum(p, e);
-}
-dd operator/(dd a, dd b) {
-    const double q1 = a.h / b.h;
-    dd r = a + -(b * dd{q1, 0.0});
-    const double q2 = r.h / b.h;
-    r = r + -(b * dd{q2, 0.0});
-    return two_sum(q1, q2) + dd{r.h / b.h, 0.0};
-}
-}  // namespace
-
-static void kb_poly64_make(int m, double beta, std::vector<double>& coef) {
-    constexpr int n = WPOLY64_ROWS;
-    const int WP = wpoly_stride(m);
-    coef.assign((size_t)n * WP, 0.0);
-    const dd hb2 = dd{0.5 * beta, 0.0} * dd{0.5 * beta, 0.0}, m2 = dd{(double)m * m, 0.0};
-    double x[n];
-    for (int k = 0; k < n; ++k) x[k] = std::cos(M_PI * (k + 0.5) / n);
-    for (int s = 1; s <= m; ++s) {
-        dd f[n];
-        for (int k = 0; k < n; ++k) {
-            // delta = (v + 1) / 2 + m - s; z = (beta / 2)^2 (1 - (delta / m)^2); I0 = sum z^i / (i!)^2
-            const dd delta = two_sum(0.5 * x[k], 0.5) + dd{(double)(m - s), 0.0};
-            const dd z = hb2 * (dd{1.0, 0.0} + -((delta * delta) / m2));
-            dd sum{1.0, 0.0}, term{1.0, 0.0};
-            for (int i = 1; i < 400; ++i) {
-                term = (term * z) / dd{(double)i * i, 0.0};
-                sum = sum + term;
-                if (std::fabs(term.h) < 1e-33 * std::fabs(sum.h)) break;
-            }
-            f[k] = sum;
-        }
-        for (int j = 1; j < n; ++j)   // divided differences
-            for (int k = n - 1; k >= j; --k) f[k] = (f[k] + -f[k - 1]) / two_sum(x[k], -x[k - j]);
-        dd c[n];
-        for (int k = 0; k < n; ++k) c[k] = dd{0.0, 0.0};
-        for (int j = n - 1; j >= 0; --j) {   // c(v) <- c(v) (v - x_j) + f_j
-            for (int k = n - 1; k >= 1; --k) c[k] = c[k - 1] + -(c[k] * dd{x[j], 0.0});
-            c[0] = -(c[0] * dd{x[j], 0.0}) + f[j];
-        }
-        for (int k = 0; k < n; ++k) coef[(size_t)k * WP + s - 1] = c[k].h;
-    }
-}
-
+// The float64 window table of (m, beta) (polytable.h).  The last tables are kept: a program's plans, and the weights'
+// inner plans, share a few windows.
 static void kb_poly64(int m, double beta, std::vector<double>& coef) {
     struct Entry { int m; double beta; std::vector<double> coef; };
     static std::mutex mu;
@@ -401,7 +349,7 @@ static void kb_poly64(int m, double beta, std::vector<double>& coef) {
         for (const Entry& e : cache)
             if (e.m == m && e.beta == beta) { coef = e.coef; return; }
     }
-    kb_poly64_make(m, beta, coef);
+    kb_poly_table<WPOLY64_ROWS>(m, beta, wpoly_stride(m), coef);
     std::lock_guard<std::mutex> lk(mu);
     cache[next] = Entry{m, beta, coef};
     next = (next + 1) % 16;
