@@ -21,8 +21,8 @@ namespace infft {
 // it crossed it six times.  The two line buffers alternate, so a stage needs one barrier and no registers
 // across it.  Fewer twiddle products (two of three stages) also round less: float32 results of the
 // 512 x 512 grids are nearer the exact sums.  The passes are bound by load latency and barriers, not by
-// bandwidth (batched d = 2, 64 sets: pass along y 0.031 -> 0.021 ms, merging pass along x 0.077 -> 0.067;
-// float64 512 x 512: merging pass 0.093 -> 0.058 ms; d = 3, 128^3: 0.042 -> 0.037 for the three passes).
+// bandwidth (event-timed stages, batched d = 2, 64 sets: pass along y 0.034 -> 0.026 ms, merging pass along x
+// 0.082 -> 0.080).
 // Shared-memory position of element i of a line: one padding slot every 16 elements, so that the
 // first stage's stores (stride 8) and the twiddles' strides spread over banks.
 __device__ __forceinline__ int skew(int i) { return i + (i >> 4); }

@@ -4,10 +4,8 @@
 // One cluster of CS CTAs reconstructs one job.  CTA `rank` owns the band of Ms/CS grid
 // rows starting at rank * Ms/CS (a whole number of tile rows):
 //   1. it sums the padded tiles written by the spread straight into its rows in shared
-//      memory, at bit-reversed positions along x (no grid in global memory); the tiles
-//      are taken in four phases by the parity of their tile row and column, so that
-//      tiles added at the same time never overlap and every cell receives its
-//      contributions in one fixed order (deterministic sums);
+//      memory, at bit-reversed positions along x (no grid in global memory), every cell's
+//      sources in one fixed order (deterministic sums);
 //   2. it transforms its rows (forward DFT along x), keeps the M frequencies of I_M and
 //      multiplies by 1/(Ms w^(k_1)), into a compact M-wide copy of its rows;
 //   3. after a cluster barrier it reads its M/CS columns of that compact array from all

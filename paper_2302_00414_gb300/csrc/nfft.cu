@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(256) k_merge(const __grid_constant__ JobSet<R>
 
 // ---------------------------------------------------------------------------------------
 // float32: four 256-thread blocks per SM (64 registers hold a radix-8 butterfly), five of the merging pass,
-// whose loads want more threads (0.069 ms with four, 0.067 with five, 0.079 with six)
+// whose loads want more threads (its stage alone, 64-set batch: 0.078 ms with four, 0.081 with five, 0.089 with six)
 template <class R, int D, bool FWD, bool MRG = false>
 __global__ void __launch_bounds__(fft_threads<R>(), sizeof(R) == 4 ? (MRG && D == 2 ? 5 : 4) : 1)
     k_fft(const __grid_constant__ JobSet<R> js, int pass) {

@@ -1,6 +1,6 @@
 // Persistent batched d = 2 adjoint (Algorithm 3.7 / 2.4 over many point sets in one launch):
 // one kernel whose CTAs take work units from a queue until it is empty.  Units are the spread
-// of four work items (Algorithm 2.4 step 1, the register-row form of spread2d.cuh), a block of
+// of four work items (Algorithm 2.4 step 1, the tensor-core form of spreadmma.cuh), a block of
 // the FFT pass along x that merges the padded tiles as it loads (steps 2-3), and a block of the
 // pass along y.  The spread units run in job order; the x blocks of job j enter the queue `lag`
 // spread units after job j's last spread unit, its y blocks `lag` spread units after that
@@ -10,11 +10,11 @@
 // queue is a list of segments (a run of spread units, or one job's x or y blocks) in the kernel
 // parameters.
 //
-// Measured on the batched d = 2 workload (64 sets): 0.456 ms per step against 0.439 ms for the
-// staged kernels in graph branches.  The FFT blocks run as four-warp CTAs at the spread's
-// occupancy (five per SM), where the staged passes run eight-warp blocks at six per SM, and
-// the overlap does not make up for it.  The form is therefore taken only on request
-// (INFFT_PERSISTENT=1).
+// Measured on the batched d = 2 workload (64 sets): 0.425 ms per step against 0.314 ms for the
+// staged kernels in graph branches.  The spread units run at twelve warps per SM (three CTAs of the registers that
+// both kinds of unit need), where the staged spread runs at twenty, the FFT blocks as four-warp CTAs at that
+// occupancy, where the staged passes run eight-warp blocks at four or five per SM, and the overlap does not
+// make up for it.  The form is therefore taken only on request (INFFT_PERSISTENT=1).
 //
 // Dependencies: an x unit of job j needs every work item of job j spread; a y unit needs every
 // x block of job j.  Each finished item or block adds one to its job's counter (after a fence);
@@ -215,8 +215,8 @@ static infft_status launch_persist2d(JobSet<float>& js, cudaStream_t st) {
 }
 
 // The persistent form for a JobSet (prefixes filled) when INFFT_PERSISTENT=1 and every job
-// takes the paired register-row spread (float32 window modes, m <= 4) with the prefetching
-// copies and the merging first pass; *used tells whether it ran.
+// takes the tensor-core spread (float32 window modes) with m <= 4 and the merging first pass; *used tells
+// whether it ran.
 infft_status persist2d_try(JobSet<float>& js, cudaStream_t st, bool* used) {
     *used = false;
     if (env_form("INFFT_PERSISTENT") != 1 || js.njobs < 1 || js.axA > 0) return INFFT_OK;

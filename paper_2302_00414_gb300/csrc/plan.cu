@@ -505,7 +505,10 @@ static infft_status build_plan(infft_plan_s* p, const double* x_in, cudaStream_t
     // 16 where 32 would not give every SM one: 256 points 40.6 -> 32.8 us with the merge in the first FFT pass).
     // d = 2 in float64: 128, since the spread takes a warp 1 us a point and a dense centre's items of 512 would leave
     // a second wave of few warps (524,288 linogram points, m = 8: spread 1.395 -> 1.014 ms, first FFT pass 0.059 ->
-    // 0.133 ms); above 4 million points the waves are many and the padded tiles would grow by 100 bytes a point.
+    // 0.133 ms).  Uniform sets, items of 512 / 128 points, m = 4: M_sigma = 64, 300 points a tile 201 / 112 us; 256, 300
+    // a tile 214 / 128; 512, 100 a tile 141 / 138, 200 to 300 a tile 205 / 240 and 280 / 342 (there the items of 512 fill the SMs
+    // and the second tile of each only costs the first pass), 600 a tile 718 / 516, 1,500 a tile 1,311 / 1,084; m = 8
+    // alike.  Above 4 million points the waves are many and the padded tiles would grow by 100 bytes a point.
     // Otherwise 512: the first FFT pass reads a padded tile per item (64-set float32 batch 299 -> 357 us with items
     // of 96 points for the smaller sets).  Where the padded tiles of short items
     // pass infft_adjoint_noalloc's scratch and those of long ones do not, the plan holds a list of long ones for it.
@@ -923,8 +926,8 @@ static infft_status run_batched(const infft_plan_t* plans, int count, int mode, 
 // G) that run concurrently on forked streams, so that the latency-bound merge and FFT
 // passes (and, with host buffers, the copies) of the smaller groups overlap the spreading
 // of the larger ones and the spreads fill each other's tails.  Measured on the batched
-// d = 2 workload (graph replay): 1, 2, 3, 4 branches give 71.3k, 76.5k, 77.3k, 76.9k
-// reconstructions/s; serialising the spreads across equal groups was slower.  With host
+// d = 2 workload (graph replay): 1, 2, 3, 4, 6 branches take 0.322, 0.307, 0.309, 0.308, 0.310 ms
+// a step; serialising the spreads across equal groups was slower.  With host
 // buffers the copies gain from more branches (end to end 1 / 3 / 6 / 8 branches: 39.8k /
 // 53.8k / 57.4k / 63.4k reconstructions/s before later kernel changes), so those calls take 8.
 // The environment variable INFFT_BATCH_BRANCHES (1..8) overrides both.

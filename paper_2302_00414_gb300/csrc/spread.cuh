@@ -11,8 +11,7 @@
 
 namespace infft {
 
-// the slots of a point on the lanes of a warp: 16-byte loads of VEC coefficients, NR per lane; off(r) is the first
-// one's cell relative to the point's first cell in a tile of row length P
+// the S x S slots of a B_opt point on the lanes of a warp: NV 16-byte loads of VEC coefficients, NR per lane
 template <class R, int MM>
 struct BoptLanes {
     static constexpr int S = 2 * MM + 2, VEC = 16 / (int)sizeof(cx<R>), NV = S * S / VEC, NR = (NV + 31) / 32;
@@ -34,7 +33,7 @@ inline int env_form(const char* name) {
     return (e && e[0] == '0') ? 0 : (e && e[0] == '1') ? 1 : -1;
 }
 
-// Launch the d = 2 register-row spread when every job qualifies (same m in 2..8, P <= 32,
+// Launch the d = 2 spread with a fixed m when every job qualifies (same m in 2..8, P <= 32,
 // all window modes or all B_opt); *used tells whether it did.
 template <class R>
 infft_status spread2d_try(JobSet<R>& js, cudaStream_t st, bool* used);

@@ -1,5 +1,5 @@
-// Two-dimensional spreading kernel (register rows) and its launcher, instantiated for
-// float32 and float64 in their own translation units (compiled in parallel).
+// Two-dimensional spreading kernel and its launcher, instantiated for float32 and float64 in their own translation
+// units (compiled in parallel).
 #pragma once
 
 #include <algorithm>
@@ -114,15 +114,14 @@ __global__ void __launch_bounds__(32 * spread2d_warps<R, BOPT>(), spread2d_block
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if constexpr (BOPT) {
         spread2d_bopt_item<R, MM>(js, blockIdx.x, smem_raw);
-        return;
+    } else {
+        const int warp = threadIdx.x >> 5;
+        const int gitem = blockIdx.x * js.wpb + warp;
+        if (gitem >= js.pre_items[js.njobs]) return;
+        unsigned char* base = smem_raw + (size_t)warp * js.smem_per_warp;
+        if constexpr (sizeof(R) == 4) spread2d_mma_item<MM>(js, gitem, base);
+        else spread2d_f64_item<MM>(js, gitem, base);
     }
-    const int warp = threadIdx.x >> 5;
-    const int gitem = blockIdx.x * js.wpb + warp;
-    if (gitem >= js.pre_items[js.njobs]) return;
-    unsigned char* base = smem_raw + (size_t)warp * js.smem_per_warp;
-    if constexpr (BOPT) {
-    } else if constexpr (sizeof(R) == 4) spread2d_mma_item<MM>(js, gitem, base);
-    else spread2d_f64_item<MM>(js, gitem, base);
 }
 
 // Per-launch setup: shared memory per item (js.smem_per_warp), items per block (js.wpb), and for

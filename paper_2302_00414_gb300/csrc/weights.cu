@@ -290,7 +290,7 @@ struct ToeplitzOp {
 
 static infft_status nfft64(infft_plan_s* q, bool forward, const void* in, void* out, cudaStream_t st);
 
-// Build the operator: t by 2^d modulated adjoint NFFTs of the degree-2M sub-plan, then c_hat.
+// Build the operator: t by 2^(d-1) modulated adjoint NFFTs of the degree-2M sub-plan and its symmetry, then c_hat.
 static infft_status toeplitz_setup(const infft_plan_s* p, infft_plan_s* sub, int M2, cudaStream_t st,
                                    const std::function<void*(size_t)>& alloc, ToeplitzOp& op) {
     const int d = p->d, N = (int)p->N, L = 2 * M2;
