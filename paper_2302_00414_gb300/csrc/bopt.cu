@@ -553,7 +553,7 @@ static infft_status optimize_impl(infft_plan_s* p, unsigned opts, double* max_re
         // a few columns do not share an SM: all threads then, for the length of the one column's chain
         const int nthr = (int)v.size() <= 2 * nsm ? BOPT_THREADS : many[k];
         int per_sm = 0;
-        INFFT_CUDA(cudaFuncSetAttribute(k_bopt_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        INFFT_TRY(smem_limit<k_bopt_solve>(smem));
         INFFT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bopt_solve, nthr, smem));
         const int blocks = nsm * std::max(1, per_sm);
         const long long chunk = 16LL * blocks;
@@ -590,7 +590,7 @@ static infft_status optimize_impl(infft_plan_s* p, unsigned opts, double* max_re
             return INFFT_ENOMEM;
         }
         const size_t smem = (fix_smem ? bopt_fixed_bytes(n_big, g.d) : 0) + 16 + 64;
-        INFFT_CUDA(cudaFuncSetAttribute(k_bopt_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        INFFT_TRY(smem_limit<k_bopt_solve>(smem));
         // one column per block per launch (largest first)
         const size_t nchunk = (big.size() + (size_t)blocks - 1) / (size_t)blocks;
         int* next = (int*)alloc(nchunk * 4);   // one work counter per launch

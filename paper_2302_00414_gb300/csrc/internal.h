@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdint>
 #include <string>
@@ -140,11 +141,37 @@ bool fault(unsigned bit);
         }                                                                                  \
     } while (0)
 
-#define INFFT_TRY(expr)                                                                    \
+#define INFFT_TRY(...)                                                                     \
     do {                                                                                   \
-        infft_status s__ = (expr);                                                         \
+        infft_status s__ = (__VA_ARGS__);                                                  \
         if (s__ != INFFT_OK) return s__;                                                   \
     } while (0)
+
+// Allow launches of kernel K with `bytes` of dynamic shared memory.  A kernel's limit is one per process and device, not
+// per launch: set to each launch's own size, one host thread lowered it between another's setting and launch, which then
+// failed.  It goes up once, to all that a block can have beside the kernel's static arrays, and stays; the launch's
+// own size alone decides what it takes and how many blocks an SM holds.
+template <auto K>
+infft_status smem_limit(size_t bytes) {
+    static std::atomic<int> limit[64];   // by device; 0: not raised yet (threads that meet here set the same value)
+    int dev = 0;
+    INFFT_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) { set_error("device %d out of range", dev); return INFFT_EINVAL; }
+    int have = limit[dev].load(std::memory_order_acquire);
+    if (have == 0) {
+        cudaFuncAttributes a;
+        INFFT_CUDA(cudaFuncGetAttributes(&a, K));
+        INFFT_CUDA(cudaDeviceGetAttribute(&have, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        have -= (int)a.sharedSizeBytes;
+        INFFT_CUDA(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, have));
+        limit[dev].store(have, std::memory_order_release);
+    }
+    if (bytes > (size_t)have) {
+        set_error("a block needs %zu bytes of shared memory, the device gives %d", bytes, have);
+        return INFFT_ECUDA;
+    }
+    return INFFT_OK;
+}
 
 infft_status dev_alloc(infft_plan_s* p, void** ptr, size_t bytes);
 // in-place exclusive prefix sum of n ints on the device (stream ordered)

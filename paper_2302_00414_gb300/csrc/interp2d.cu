@@ -106,7 +106,7 @@ static infft_status launch_interp_bopt2d(JobSet<R>& js, cudaStream_t st) {
     const size_t smem = (size_t)P * P * sizeof(cx<R>);
     const int nitems = js.pre_items[js.njobs];
     if (nitems == 0) return INFFT_OK;
-    INFFT_CUDA(cudaFuncSetAttribute(k_interp_bopt2d<R, MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    INFFT_TRY(smem_limit<k_interp_bopt2d<R, MM>>(smem));
     k_interp_bopt2d<R, MM><<<nitems, 32 * INTERP_BOPT_WARPS, smem, st>>>(js);
     INFFT_LAUNCHED();
     return INFFT_OK;

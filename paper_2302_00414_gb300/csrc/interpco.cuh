@@ -148,7 +148,7 @@ static infft_status launch_interp_co(JobSet<float>& js, cudaStream_t st) {
     const size_t smem = InterpCo<MM>::bytes(P);
     const int nitems = js.pre_items[js.njobs];
     if (nitems == 0) return INFFT_OK;
-    INFFT_CUDA(cudaFuncSetAttribute(k_interp_co<MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    INFFT_TRY(smem_limit<k_interp_co<MM>>(smem));
     INFFT_CUDA(cudaFuncSetAttribute(k_interp_co<MM>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     (int)cudaSharedmemCarveoutMaxShared));
     k_interp_co<MM><<<nitems, 32 * INTERP_CO_WARPS, smem, st>>>(js);

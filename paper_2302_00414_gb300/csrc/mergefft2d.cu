@@ -264,7 +264,7 @@ template <class R, int CS>
 static infft_status mf_launch(const JobSet<R>& js, const JobSel& sel, size_t smem, cudaStream_t st, bool* ok) {
     *ok = false;
     auto kern = k_mergefft2d<R, CS>;
-    INFFT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    INFFT_TRY(smem_limit<k_mergefft2d<R, CS>>(smem));
     if (CS > 8) INFFT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sel.n * CS));

@@ -436,7 +436,7 @@ static JobSet<R>* new_subset(const JobSet<R>& js, const std::vector<int>& idx) {
 template <class R, int D>
 static infft_status launch_fft_adjoint(JobSet<R>& js, cudaStream_t st, cudaEvent_t* ev) {
     const size_t fsmem = fft_smem(js);
-    INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+    INFFT_TRY(smem_limit<k_fft<R, D, false>>(fsmem));
     for (int p = 0; p < D; ++p) {
         k_fft<R, D, false><<<js.pre_fft[p][js.njobs], fft_threads<R>(), fsmem, st>>>(js, p);
         INFFT_LAUNCHED();
@@ -448,12 +448,12 @@ static infft_status launch_fft_adjoint(JobSet<R>& js, cudaStream_t st, cudaEvent
 template <class R>
 static infft_status launch_fft_adjoint_mrg(JobSet<R>& js, cudaStream_t st, cudaEvent_t* ev) {
     const size_t msmem = fft_smem_mrg(js);
-    INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 2, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msmem));
+    INFFT_TRY(smem_limit<k_fft<R, 2, false, true>>(msmem));
     k_fft<R, 2, false, true><<<js.pre_fft[0][js.njobs], fft_threads<R>(), msmem, st>>>(js, 0);
     INFFT_LAUNCHED();
     if (ev) INFFT_CUDA(cudaEventRecord(ev[3], st));
     const size_t fsmem = fft_smem(js);
-    INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+    INFFT_TRY(smem_limit<k_fft<R, 2, false>>(fsmem));
     k_fft<R, 2, false><<<js.pre_fft[1][js.njobs], fft_threads<R>(), fsmem, st>>>(js, 1);
     INFFT_LAUNCHED();
     if (ev) INFFT_CUDA(cudaEventRecord(ev[4], st));
@@ -530,7 +530,7 @@ static infft_status launch_adjoint(JobSet<R>& js, cudaStream_t st, cudaEvent_t* 
     const int nitems = js.pre_items[js.njobs];
     if (nitems > 0) {
         const size_t smem = spw * js.wpb;
-        INFFT_CUDA(cudaFuncSetAttribute(k_spread<R, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        INFFT_TRY(smem_limit<k_spread<R, D>>(smem));
         k_spread<R, D><<<(nitems + js.wpb - 1) / js.wpb, 32 * js.wpb, smem, st>>>(js);
         INFFT_LAUNCHED();
     }
@@ -545,7 +545,7 @@ static infft_status launch_adjoint(JobSet<R>& js, cudaStream_t st, cudaEvent_t* 
         if (on_load) {
             if (ev) INFFT_CUDA(cudaEventRecord(ev[2], st));
             const size_t fsmem = fft_smem(js);
-            INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 1, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+            INFFT_TRY(smem_limit<k_fft<R, 1, false, true>>(fsmem));
             k_fft<R, 1, false, true><<<js.pre_fft[0][js.njobs], fft_threads<R>(), fsmem, st>>>(js, 0);
             INFFT_LAUNCHED();
             if (ev) INFFT_CUDA(cudaEventRecord(ev[3], st));
@@ -563,7 +563,7 @@ template <class R, int D>
 static infft_status launch_forward(JobSet<R>& js, cudaStream_t st) {
     fill_prefixes(js, D, true);
     const size_t fsmem = fft_smem(js);
-    INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+    INFFT_TRY(smem_limit<k_fft<R, D, true>>(fsmem));
     for (int p = 0; p < D; ++p) {
         k_fft<R, D, true><<<js.pre_fft[p][js.njobs], fft_threads<R>(), fsmem, st>>>(js, p);
         INFFT_LAUNCHED();
@@ -590,7 +590,7 @@ static infft_status launch_forward(JobSet<R>& js, cudaStream_t st) {
     const int nitems = js.pre_items[js.njobs];
     if (nitems > 0) {
         const size_t smem = spw * js.wpb;
-        INFFT_CUDA(cudaFuncSetAttribute(k_interp<R, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        INFFT_TRY(smem_limit<k_interp<R, D>>(smem));
         k_interp<R, D><<<(nitems + js.wpb - 1) / js.wpb, 32 * js.wpb, smem, st>>>(js);
         INFFT_LAUNCHED();
     }
@@ -629,13 +629,13 @@ static infft_status fft_passes_d(JobSet<R>& js, cudaStream_t st, bool forward) {
     const int n = js.job[0].Ms;
     const size_t fsmem = fft_smem(js);
     if (forward) {
-        INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+        INFFT_TRY(smem_limit<k_fft<R, D, true>>(fsmem));
         for (int p = 0; p < D; ++p) {
             k_fft<R, D, true><<<js.pre_fft[p][1], fft_threads<R>(), fsmem, st>>>(js, p);
             INFFT_LAUNCHED();
         }
     } else {
-        INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+        INFFT_TRY(smem_limit<k_fft<R, D, false>>(fsmem));
         for (int p = 0; p < D; ++p) {
             k_fft<R, D, false><<<js.pre_fft[p][1], fft_threads<R>(), fsmem, st>>>(js, p);
             INFFT_LAUNCHED();
@@ -675,7 +675,7 @@ infft_status run_fft_axis(const Job<R>& J, long long A, long long B, int nblk, c
     }
     js.pre_fft[0][1] = (int)((lines + js.L - 1) / js.L);
     const size_t fsmem = fft_smem(js);
-    INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem));
+    INFFT_TRY(smem_limit<k_fft<R, 2, false>>(fsmem));
     k_fft<R, 2, false><<<js.pre_fft[0][1], fft_threads<R>(), fsmem, st>>>(js, 0);
     INFFT_LAUNCHED();
     return INFFT_OK;
@@ -709,15 +709,15 @@ static infft_status fft_conv_d(const Job<R>& J, cudaStream_t st) {
     fill_prefixes(ja, D, false);
     const size_t smem = fft_smem(js);
     for (int p = 0; p + 1 < D; ++p) {
-        INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        INFFT_TRY(smem_limit<k_fft<R, D, true>>(smem));
         k_fft<R, D, true><<<js.pre_fft[p][1], fft_threads<R>(), smem, st>>>(js, p);
         INFFT_LAUNCHED();
     }
-    INFFT_CUDA(cudaFuncSetAttribute(k_fft_conv<R, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    INFFT_TRY(smem_limit<k_fft_conv<R, D>>(smem));
     k_fft_conv<R, D><<<ja.pre_fft[0][1], fft_threads<R>(), smem, st>>>(ja);
     INFFT_LAUNCHED();
     for (int p = 1; p < D; ++p) {
-        INFFT_CUDA(cudaFuncSetAttribute(k_fft<R, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        INFFT_TRY(smem_limit<k_fft<R, D, false>>(smem));
         k_fft<R, D, false><<<ja.pre_fft[p][1], fft_threads<R>(), smem, st>>>(ja, p);
         INFFT_LAUNCHED();
     }

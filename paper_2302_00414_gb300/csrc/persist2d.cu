@@ -193,7 +193,7 @@ static infft_status launch_persist2d(JobSet<float>& js, cudaStream_t st) {
     spread2d_setup<float, MM, false>(js);
     const size_t smem = std::max({(size_t)4 * js.smem_per_warp, fft_smem_mrg(js), fft_smem(js)});
     auto kern = k_adjoint2d_persistent<MM>;
-    INFFT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    INFFT_TRY(smem_limit<k_adjoint2d_persistent<MM>>(smem));
     int dev = 0, nsm = 0, per_sm = 0;
     INFFT_CUDA(cudaGetDevice(&dev));
     INFFT_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

@@ -224,7 +224,7 @@ static infft_status launch_spread3d_m(JobSet<R>& js, cudaStream_t st) {
     const int nitems = js.pre_items[js.njobs];
     if (nitems == 0) return INFFT_OK;
     const size_t smem = spw * js.wpb;
-    INFFT_CUDA(cudaFuncSetAttribute(k_spread3d<R, MM, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    INFFT_TRY(smem_limit<k_spread3d<R, MM, PF>>(smem));
     // the tiles bound the warps per SM: ask for all of the SM's unified memory as shared memory
     INFFT_CUDA(cudaFuncSetAttribute(k_spread3d<R, MM, PF>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     (int)cudaSharedmemCarveoutMaxShared));

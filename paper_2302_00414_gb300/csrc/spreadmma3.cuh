@@ -220,7 +220,7 @@ static infft_status launch_spread3d_mma(JobSet<float>& js, cudaStream_t st) {
     const int nitems = js.pre_items[js.njobs];
     if (nitems == 0) return INFFT_OK;
     const int smem = SpreadMma3<MM>::BYTES;
-    INFFT_CUDA(cudaFuncSetAttribute(k_spread3d_mma<MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    INFFT_TRY(smem_limit<k_spread3d_mma<MM>>(smem));
     INFFT_CUDA(cudaFuncSetAttribute(k_spread3d_mma<MM>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     (int)cudaSharedmemCarveoutMaxShared));
     k_spread3d_mma<MM><<<nitems, 64, smem, st>>>(js);
