@@ -57,43 +57,61 @@ __device__ __forceinline__ R kb_phi(R delta, R inv_m, R beta) {
     return (s >= R(0)) ? bessel_i0(beta * sqrt(s)) : R(0);
 }
 
-// centred cardinal B-spline of order 2m evaluated at delta (grid units), by the
-// Cox-de Boor recursion on the uniform knots -m..m; used for the B-spline window
-// (eq. window_bspline).  Only small orders are supported (2m <= 16).
-template <class R>
-__device__ __forceinline__ R bspline_phi(R delta, int m) {
-    const int n = 2 * m;
-    R y = delta + R(m);  // shift to [0, n)
-    if (!(y >= R(0) && y < R(n))) return R(0);
-    R b[17];
-    int cell = (int)floor(y);
-    for (int i = 0; i < n; ++i) b[i] = (i == cell) ? R(1) : R(0);
-    for (int k = 1; k < n; ++k) {
-        for (int i = 0; i < n - k; ++i) {
-            R left = (y - R(i)) / R(k);
-            R right = (R(i + k + 1) - y) / R(k);
-            b[i] = left * b[i] + right * b[i + 1];
-        }
-    }
-    return b[0];
-}
-
 enum WindowKind { WK_KB = 0, WK_BSPLINE = 1, WK_DIRICHLET = 2 };
-
-template <class R>
-__device__ __forceinline__ R window_phi(int kind, R delta, int m, R inv_m, R beta) {
-    if (kind == WK_BSPLINE) return bspline_phi<R>(delta, m);
-    return kb_phi<R>(delta, inv_m, beta);
-}
 
 // Window value of tap s = 0..2m of a point with fractional offset u = M_sigma x - b in
 // [0, 1] (b = floor(M_sigma x)); the tap sits at l = b - m + s, delta = u + m - s.
 // Membership in the index set (eq. indexset_x) is decided exactly: taps 1..2m always
 // satisfy |delta| <= m, tap 0 only when u = 0 (the point on a grid node).
 template <class R>
-__device__ __forceinline__ R tap_weight(int kind, R u, int s, int m, R inv_m, R beta) {
+__device__ __forceinline__ R kb_tap(R u, int s, int m, R inv_m, R beta) {
     if (s == 0 && u != R(0)) return R(0);
-    return window_phi<R>(kind, u + R(m - s), m, inv_m, beta);
+    return kb_phi<R>(u + R(m - s), inv_m, beta);
+}
+
+// The taps of the centred cardinal B-spline of order n = 2m (eq. window_bspline; 2m <= 16) by the Cox-de Boor
+// recursion on the uniform knots -m..m, once for all taps: with w_j the value at u + j above the first knot,
+//   order k + 1:  w_j <- (u + j) w_j + (k + 1 - j - u) w_{j-1}
+// without the 1 / k of each order, which is 1 / (n - 1)! at the end.  All terms are positive: no digits are lost.
+// Tap s is w_{2m-s}; tap 0, on a node, is zero.  (A recursion for each tap by itself takes 2m times the work: where a
+// kernel stages few points at a time, sparse d = 3 sets in float32, it was three quarters of the call.)
+template <int MM, class R>
+__device__ __forceinline__ void bspline_taps(R u, R* out) {
+    constexpr int n = 2 * MM;
+    R w[n];
+    w[0] = R(1);
+    double fact = 1;
+#pragma unroll
+    for (int k = 1; k < n; ++k) {
+        fact *= k;
+        w[k] = (R(1) - u) * w[k - 1];
+#pragma unroll
+        for (int j = n - 1; j >= 1; --j)
+            if (j < k) w[j] = fma(u + R(j), w[j], (R(k + 1 - j) - u) * w[j - 1]);
+        w[0] *= u;
+    }
+    // 1 / (n - 1)! to twice the precision: rounded, it would scale every value alike
+    const double inv = 1.0 / fact;
+    const R hi = R(inv), lo = R(sizeof(R) == 4 ? inv - (double)hi : fma(-inv, fact, 1.0) * inv);
+    out[0] = R(0);
+#pragma unroll
+    for (int s = 1; s <= n; ++s) out[s] = fma(w[n - s], hi, w[n - s] * lo);
+}
+// for m known at run time only; out[0..2m] holds the triangle
+template <class R>
+__device__ __forceinline__ void bspline_taps_any(int m, R u, R* out) {
+    const int n = 2 * m;
+    R fact = R(1);
+    out[n] = R(1);
+    for (int k = 1; k < n; ++k) {
+        fact *= R(k);
+        R* w = out + n;   // w_j at w[-j]
+        w[-k] = (R(1) - u) * w[1 - k];
+        for (int j = k - 1; j >= 1; --j) w[-j] = fma(u + R(j), w[-j], (R(k + 1 - j) - u) * w[1 - j]);
+        w[0] *= u;
+    }
+    out[0] = R(0);
+    for (int s = 1; s <= n; ++s) out[s] /= fact;
 }
 
 // Float32 plans evaluate the Kaiser-Bessel taps s = 1..2m from per-plan polynomials:
@@ -219,6 +237,14 @@ __device__ __forceinline__ void poly_taps_any(const R* __restrict__ c, int m, R 
     out[0] = (u == R(0)) ? R(1) : R(0);
 }
 
+// the 2m + 1 taps of a job's window for m known at run time only
+template <class R>
+__device__ __forceinline__ void taps_any(int window, const R* __restrict__ wpoly, int m, R inv_m, R beta, R u, R* out) {
+    if (window == WK_BSPLINE) bspline_taps_any<R>(m, u, out);
+    else if (wpoly) poly_taps_any<R>(wpoly, m, u, out);
+    else for (int s = 0; s <= 2 * m; ++s) out[s] = kb_tap<R>(u, s, m, inv_m, beta);
+}
+
 // ----------------------------------------------------------------------------------------
 // Work descriptors.  One Job describes one transform (one plan, one in/out pair);
 // kernels receive an array of Jobs with the same d and precision and map their
@@ -242,7 +268,7 @@ struct Job {
     const int* tile_items;     // ntile^d + 1 prefix of items per tile
     const int* cell_start;     // sorted position of each cell's first point, cells tile-major
     const R* dinv;             // M entries 1/(Ms w^(k)) (per axis); float32: then their low parts
-    const R* wpoly;            // wpoly_rows x wpoly_stride(m) window polynomial (Kaiser-Bessel plans) or null
+    const R* wpoly;            // wpoly_rows x wpoly_stride(m) window polynomial (Kaiser-Bessel; float32 B-spline) or null
     const float* wpoly_h;      // host copy of the same table (read by the launchers only) or null
     const cx<R>* tw;           // Ms/2 twiddles exp(-2 pi i k / Ms); float32: then their low parts
     cx<R>* padded;             // nitems * P^d

@@ -42,7 +42,7 @@ struct infft_plan_s {
     void* dinv = nullptr;     // M entries
     void* tw = nullptr;       // Ms/2 complex
     void* dinv_win = nullptr; // M entries for the B_opt window (may alias dinv)
-    void* wpoly = nullptr;    // window polynomial table (Kaiser-Bessel plans, plan precision)
+    void* wpoly = nullptr;    // window polynomial table (Kaiser-Bessel plans, plan precision; float32 B-spline plans)
     std::vector<float> wpoly_host;   // host copy of the float32 table
 
     // weights (device): caller order float64 master + sorted copy in plan precision

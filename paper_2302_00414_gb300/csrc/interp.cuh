@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(128) k_interp_t(const __grid_constant__ JobSet
     unsigned char* base = smem_raw + (size_t)warp * js.smem_per_warp;
     cx<R>* pad = reinterpret_cast<cx<R>*>(base);
     R* poly = reinterpret_cast<R*>(pad + ((cells + 1) & ~1));
-    const bool use_poly = J.wpoly != nullptr;
+    const bool use_poly = J.window == WK_KB;
     if (use_poly) {
         for (int e = lane; e < wpoly_rows<R>() * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
     }
@@ -62,9 +62,7 @@ __global__ void __launch_bounds__(128) k_interp_t(const __grid_constant__ JobSet
             poly_taps<MM, D>(poly, uu, wt);
         } else {
 #pragma unroll
-            for (int s = 0; s < W; ++s)
-#pragma unroll
-                for (int a = 0; a < D; ++a) wt[a][s] = tap_weight<R>(J.window, uu[a], s, MM, J.inv_m, J.beta);
+            for (int a = 0; a < D; ++a) bspline_taps<MM>(uu[a], wt[a]);
         }
         const R *wz = wt[0], *wy = wt[D - 2], *wx = wt[D - 1];
         cx<R> acc = mk<R>(0, 0);

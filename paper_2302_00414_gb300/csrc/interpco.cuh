@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(32 * INTERP_CO_WARPS) k_interp_co(const __grid
     int2* sm = reinterpret_cast<int2*>(smem_raw + warp * C::PER_WARP + 32 * C::TAPS * 4);
     float* poly = reinterpret_cast<float*>(smem_raw + C::OFF_POLY);
     float2* pad = reinterpret_cast<float2*>(smem_raw + C::OFF_PAD);
-    const bool use_poly = J.wpoly != nullptr;
+    const bool use_poly = J.window == WK_KB;
     if (use_poly)
         for (int e = threadIdx.x; e < WPOLY_ROWS * wpoly_stride(MM); e += 32 * NW) poly[e] = J.wpoly[e];
     const int tz = item.x / (nt * nt), ty = (item.x / nt) % nt, tx = item.x % nt;
@@ -87,9 +87,7 @@ __global__ void __launch_bounds__(32 * INTERP_CO_WARPS) k_interp_co(const __grid
             if (use_poly) poly_taps<MM, D>(poly, u, wt);
             else {
 #pragma unroll
-                for (int s = 0; s < W; ++s)
-#pragma unroll
-                    for (int a = 0; a < D; ++a) wt[a][s] = tap_weight<float>(J.window, u[a], s, MM, J.inv_m, J.beta);
+                for (int a = 0; a < D; ++a) bspline_taps<MM>(u[a], wt[a]);
             }
 #pragma unroll
             for (int a = 0; a < D; ++a)

@@ -76,8 +76,7 @@ __global__ void __launch_bounds__(128) k_spread(const __grid_constant__ JobSet<R
                 for (int t = 0; t < D; ++t) {
                     const R u = J.u[(size_t)i * D + t];
                     R* ps = psi + (lane * D + t) * W;
-                    if (J.wpoly) poly_taps_any<R>(J.wpoly, m, u, ps);
-                    else for (int s = 0; s < W; ++s) ps[s] = tap_weight<R>(J.window, u, s, m, J.inv_m, J.beta);
+                    taps_any<R>(J.window, J.wpoly, m, J.inv_m, J.beta, u, ps);
                 }
             }
         }
@@ -349,8 +348,7 @@ __global__ void __launch_bounds__(128) k_interp(const __grid_constant__ JobSet<R
             if (!bopt) {
                 for (int t = 0; t < D; ++t) {
                     const R u = J.u[(size_t)i * D + t];
-                    if (J.wpoly) poly_taps_any<R>(J.wpoly, m, u, ps + t * W);
-                    else for (int s = 0; s < W; ++s) ps[t * W + s] = tap_weight<R>(J.window, u, s, m, J.inv_m, J.beta);
+                    taps_any<R>(J.window, J.wpoly, m, J.inv_m, J.beta, u, ps + t * W);
                 }
             }
             const cx<R>* cf = bopt ? J.coef + (size_t)i * ntap : nullptr;

@@ -564,13 +564,16 @@ static infft_status build_plan(infft_plan_s* p, const double* x_in, cudaStream_t
                                                          (cx<float>*)p->tw);
     INFFT_LAUNCHED();
 
-    // window polynomials (Kaiser-Bessel plans)
-    if (p->window == WK_KB && 2 * m + 1 <= 32) {
+    // window polynomials: Kaiser-Bessel plans, and the float32 B-spline's for the spreads on the tensor cores
+    if ((p->window == WK_KB && 2 * m + 1 <= 32) || (p->window == WK_BSPLINE && !p->fp64)) {
         const size_t n = (size_t)(p->fp64 ? WPOLY64_ROWS : WPOLY_ROWS) * wpoly_stride(m);
         INFFT_TRY(dev_alloc(p, &p->wpoly, n * R_sz));
         if (p->fp64) {
             kb_poly64(m, p->beta, wpoly64);
             INFFT_CUDA(cudaMemcpyAsync(p->wpoly, wpoly64.data(), n * R_sz, cudaMemcpyHostToDevice, st));
+        } else if (p->window == WK_BSPLINE) {
+            bspline_poly_table<WPOLY_DEG + 1>(m, wpoly_stride(m), p->wpoly_host);
+            INFFT_CUDA(cudaMemcpyAsync(p->wpoly, p->wpoly_host.data(), n * R_sz, cudaMemcpyHostToDevice, st));
         } else {
             k_wpoly<<<1, 32, 0, st>>>(m, p->beta, (float*)p->wpoly);
             INFFT_LAUNCHED();

@@ -1,9 +1,11 @@
-// Window polynomials for float64 Kaiser-Bessel plans, on the host in double-double arithmetic (Dekker / Knuth
+// Window polynomials made on the host (no CUDA header is needed).
+//
+// For float64 Kaiser-Bessel plans, in double-double arithmetic (Dekker / Knuth
 // error-free sums and products): tap s = 1..m is interpolated at n Chebyshev points of v, phi from the power series
 // of I0, and rewritten in powers of v.  What is alike for every window (the change of basis, the series' reciprocals) is
 // made once per process, 0.1 ms; a new window then takes 0.01 ms (m = 4) to 0.1 ms (m = 15) of a Grace core, a tap's nodes
 // evaluated together.  With one node after the other, a division per term and Newton's form per tap it was 0.2 to
-// 1.2 ms, beside the 0.3 to 0.4 ms of a small plan.  No CUDA header is needed.
+// 1.2 ms, beside the 0.3 to 0.4 ms of a small plan.
 #pragma once
 
 #include <algorithm>
@@ -90,6 +92,45 @@ inline void kb_poly_table(int m, double beta, int stride, std::vector<double>& c
         for (int j = 0; j < n; ++j)
             for (int k = 0; k < n; ++k) c[k] = c[k] + B.map[j][k] * f[j];
         for (int k = 0; k < n; ++k) coef[(size_t)k * stride + s - 1] = c[k].h;
+    }
+}
+
+// The float32 table of the centred cardinal B-spline of order 2m: tap s at u in [0, 1] in powers of v = 2u - 1 up to
+// v^(n - 1), coef[k stride + s - 1] for k < n, then what rounding took from k = 0.  The spline is a polynomial of degree
+// 2m - 1 there: itself for n >= 2m, else its Chebyshev interpolant (m = 8, n = 11: off by less than 1e-11 of the
+// largest value).
+template <int n>
+inline void bspline_poly_table(int m, int stride, std::vector<float>& coef) {
+    coef.assign((size_t)(n + 1) * stride, 0.f);
+    double node[n], f[n][17];   // values of every tap at the nodes, by the recursion of bspline_taps
+    for (int k = 0; k < n; ++k) {
+        node[k] = std::cos(M_PI * (k + 0.5) / n);
+        const double u = 0.5 * (node[k] + 1.0);
+        double w[16] = {1.0}, fact = 1.0;
+        for (int o = 1; o < 2 * m; ++o) {
+            fact *= o;
+            w[o] = (1.0 - u) * w[o - 1];
+            for (int j = o - 1; j >= 1; --j) w[j] = (u + j) * w[j] + (o + 1 - j - u) * w[j - 1];
+            w[0] *= u;
+        }
+        for (int s = 1; s <= 2 * m; ++s) f[k][s] = w[2 * m - s] / fact;
+    }
+    for (int s = 1; s <= m; ++s) {
+        double a[n] = {0.0}, t0[n] = {1.0}, t1[n] = {0.0, 1.0};   // powers of the sum, of T_(j-1) and of T_j
+        for (int j = 0; j < n; ++j) {
+            double c = 0.0;
+            for (int k = 0; k < n; ++k) c += f[k][s] * std::cos(j * M_PI * (k + 0.5) / n);
+            c *= (j == 0 ? 1.0 : 2.0) / n;
+            const double* t = j == 0 ? t0 : t1;
+            for (int k = 0; k < n; ++k) a[k] += c * t[k];
+            if (j >= 1) {
+                double t2[n];
+                for (int k = 0; k < n; ++k) t2[k] = -t0[k] + (k > 0 ? 2.0 * t1[k - 1] : 0.0);
+                for (int k = 0; k < n; ++k) { t0[k] = t1[k]; t1[k] = t2[k]; }
+            }
+        }
+        for (int k = 0; k < n; ++k) coef[(size_t)k * stride + s - 1] = (float)a[k];
+        coef[(size_t)n * stride + s - 1] = (float)(a[0] - (double)(float)a[0]);
     }
 }
 

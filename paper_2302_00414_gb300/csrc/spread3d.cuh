@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(64) k_spread3d(const __grid_constant__ JobSet<
     R* psx = psz + CH * WE;                                            // [CH][WE]
     int* meta = reinterpret_cast<int*>(psx + CH * WE);                 // [CH] base cell in the shared tile
     R* poly = reinterpret_cast<R*>(meta + CH);                 // window polynomial (float32 plans)
-    const bool use_poly = J.wpoly != nullptr;
+    const bool use_poly = J.window == WK_KB;
     if (use_poly) {
         for (int e = lane; e < wpoly_rows<R>() * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e];
     }
@@ -134,12 +134,9 @@ __global__ void __launch_bounds__(64) k_spread3d(const __grid_constant__ JobSet<
                 const R uu[3] = {uz, uy, ux};
                 poly_taps<MM, 3>(poly, uu, wt);
             } else {
-#pragma unroll
-                for (int s = 0; s < W; ++s) {
-                    wt[0][s] = tap_weight<R>(J.window, uz, s, MM, J.inv_m, J.beta);
-                    wt[1][s] = tap_weight<R>(J.window, uy, s, MM, J.inv_m, J.beta);
-                    wt[2][s] = tap_weight<R>(J.window, ux, s, MM, J.inv_m, J.beta);
-                }
+                bspline_taps<MM>(uz, wt[0]);
+                bspline_taps<MM>(uy, wt[1]);
+                bspline_taps<MM>(ux, wt[2]);
             }
 #pragma unroll
             for (int s = 0; s < W; ++s) {

@@ -47,7 +47,7 @@ __device__ __forceinline__ void spread2d_f64_item(const JobSet<double>& js, cons
     const int ty = item.x / J.ntile, tx = item.x % J.ntile;
     const int logMs = 31 - __clz(Ms);
     const bool dcf = J.mode == INFFT_MODE_DCF;
-    const bool use_poly = J.wpoly != nullptr;
+    const bool use_poly = J.window == WK_KB;
     double* sy = reinterpret_cast<double*>(base + C::OFF_Y);
     double* sx = reinterpret_cast<double*>(base + C::OFF_X);
     double2* sc = reinterpret_cast<double2*>(base + C::OFF_C);
@@ -92,10 +92,7 @@ __device__ __forceinline__ void spread2d_f64_item(const JobSet<double>& js, cons
                 double wt[1][W];
                 const double v = a == 0 ? u.x : u.y;
                 if (use_poly) poly_taps<MM, 1>(poly, &v, wt);
-                else {
-#pragma unroll
-                    for (int s = 0; s < W; ++s) wt[0][s] = tap_weight<double>(J.window, v, s, MM, J.inv_m, J.beta);
-                }
+                else bspline_taps<MM>(v, wt[0]);
                 double* dst = (a == 0 ? sy : sx) + lane * W;
 #pragma unroll
                 for (int s = 0; s < W; ++s) dst[s] = wt[0][s];

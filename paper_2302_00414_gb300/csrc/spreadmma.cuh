@@ -124,10 +124,9 @@ __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const
     const int ty = item.x / J.ntile, tx = item.x % J.ntile;
     const int logMs = 31 - __clz(Ms);
     const bool dcf = J.mode == INFFT_MODE_DCF;
-    const bool use_poly = J.wpoly != nullptr;
     float* poly = reinterpret_cast<float*>(base + C::OFF_POLY);
-    const float wscale = spread_mma_wscale(J.wexp);
-    if (use_poly && !js.wtab_ok)
+    const float wscale = spread_mma_wscale(J.wexp), wscale0 = J.window == WK_BSPLINE ? 0.f : wscale;   // tap 0's: on a node
+    if (!js.wtab_ok)
         for (int e = lane; e < WPOLY_ROWS * wpoly_stride(MM); e += 32) poly[e] = J.wpoly[e] * wscale;
     for (int e = lane; e < C::OFF_META / 16; e += 32) reinterpret_cast<uint4*>(base)[e] = make_uint4(0, 0, 0, 0);
     __syncwarp();   // before lanes read others' rows of the table and store taps over slots others cleared
@@ -174,23 +173,15 @@ __device__ __forceinline__ void spread2d_mma_item(const JobSet<float>& js, const
         if (c + lane < item.z) f = __ldg(reinterpret_cast<const float2*>(J.in) + perm);
     };
     auto taps = [&](float2 v, float (*wt)[W]) {   // of both coordinates, scaled to at most 2^13
-        if (use_poly) {
-            const float vv[2] = {v.x, v.y};
-            if (js.wtab_ok) {
-                poly_taps<MM, 1>(js.wtab, vv, wt);
-                poly_taps<MM, 1>(js.wtab, vv + 1, wt + 1);
-            } else {
-                poly_taps<MM, 2>(poly, vv, wt);
-            }
-            wt[0][0] *= wscale;
-            wt[1][0] *= wscale;
+        const float vv[2] = {v.x, v.y};
+        if (js.wtab_ok) {
+            poly_taps<MM, 1>(js.wtab, vv, wt);
+            poly_taps<MM, 1>(js.wtab, vv + 1, wt + 1);
         } else {
-#pragma unroll
-            for (int s = 0; s < W; ++s) {
-                wt[0][s] = wscale * tap_weight<float>(J.window, v.x, s, MM, J.inv_m, J.beta);
-                wt[1][s] = wscale * tap_weight<float>(J.window, v.y, s, MM, J.inv_m, J.beta);
-            }
+            poly_taps<MM, 2>(poly, vv, wt);
         }
+        wt[0][0] *= wscale0;
+        wt[1][0] *= wscale0;
     };
     load_point(0);
     load_sample(0);

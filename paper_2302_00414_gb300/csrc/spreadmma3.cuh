@@ -47,12 +47,11 @@ __global__ void __launch_bounds__(64, 6) k_spread3d_mma(const __grid_constant__ 
     const int tz = item.x / (nt * nt), ty = (item.x / nt) % nt, tx = item.x % nt;
     const int logMs = 31 - __clz(Ms);
     const bool dcf = J.mode == INFFT_MODE_DCF;
-    const bool use_poly = J.wpoly != nullptr;
     unsigned char* own = smem + warp * C::HALF;       // the half chunk this warp stages
     float* poly = reinterpret_cast<float*>(smem + C::OFF_POLY);
     const float wscale = spread_mma_wscale(J.wexp);   // window to at most 2^13
-    if (use_poly)
-        for (int e = threadIdx.x; e < WPOLY_ROWS * wpoly_stride(MM); e += 64) poly[e] = J.wpoly[e] * wscale;
+    const float wscale0 = J.window == WK_BSPLINE ? 0.f : wscale;   // tap 0's: on a node
+    for (int e = threadIdx.x; e < WPOLY_ROWS * wpoly_stride(MM); e += 64) poly[e] = J.wpoly[e] * wscale;
     for (int e = lane; e < C::OFF_META / 16; e += 32) reinterpret_cast<uint4*>(own)[e] = make_uint4(0, 0, 0, 0);
     __syncthreads();
 
@@ -132,13 +131,8 @@ __global__ void __launch_bounds__(64, 6) k_spread3d_mma(const __grid_constant__ 
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 float wt[1][W];
-                if (use_poly) {
-                    poly_taps<MM, 1>(poly, uu + a, wt);
-                    wt[0][0] *= wscale;
-                } else {
-#pragma unroll
-                    for (int s = 0; s < W; ++s) wt[0][s] = wscale * tap_weight<float>(J.window, uu[a], s, MM, J.inv_m, J.beta);
-                }
+                poly_taps<MM, 1>(poly, uu + a, wt);
+                wt[0][0] *= wscale0;
 #pragma unroll
                 for (int s = 0; s < W; ++s) {
                     if (a == 0) {

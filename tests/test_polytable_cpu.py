@@ -79,3 +79,39 @@ def test_cost_of_a_new_window(program):
     """A plan with a new window makes its table while the program waits: the best of 30 takes a fraction of the 0.4 ms
     that a small float64 plan takes besides."""
     assert _run(program, 8, 8 * math.pi * 1.5)[0] < 2.5e-4
+
+
+SPLINE = r"""
+#include "polytable.h"
+#include <cstdio>
+#include <cstdlib>
+int main(int argc, char** argv) {
+    std::vector<float> c;
+    infft::bspline_poly_table<11>(atoi(argv[1]), 8, c);
+    for (float v : c) printf("%.9g\n", v);
+}
+"""
+
+
+@pytest.mark.parametrize("m", range(1, 9))
+def test_float32_spline_table(m, tmp_path):
+    """The polynomials against the B-spline in rational arithmetic: the coefficients' float32 rounding, half a unit each
+    (the constant's low part is in the table), and 1e-11 of the largest value for order 16 in degree 10."""
+    from fractions import Fraction
+    cc = shutil.which("g++")
+    if cc is None:
+        pytest.skip("no host compiler")
+    (tmp_path / "s.cpp").write_text(SPLINE)
+    subprocess.run([cc, "-O2", "-std=c++17", "-I", CSRC, str(tmp_path / "s.cpp"), "-o", str(tmp_path / "s")], check=True)
+    out = subprocess.run([str(tmp_path / "s"), str(m)], capture_output=True, text=True, check=True).stdout.split()
+    c = [float(v) for v in out]
+    n = 2 * m
+    for s in range(1, m + 1):
+        col = [c[8 * k + s - 1] for k in range(12)]
+        bound = 2.0 ** -24 * sum(abs(v) for v in col[1:11]) + 2.0 ** -47 * abs(col[0]) + 1e-11
+        for u in (Fraction(0), Fraction(1, 7), Fraction(1, 2), Fraction(15, 16), Fraction(1)):
+            y = u + m - s + Fraction(n, 2)
+            ref = sum((-1) ** k * math.comb(n, k) * (y - k) ** (n - 1) for k in range(n + 1) if y > k) / math.factorial(n - 1)
+            v = 2 * u - 1
+            p = sum(Fraction(col[k]) * v ** k for k in range(11)) + Fraction(col[11])
+            assert abs(float(p - ref)) <= bound
