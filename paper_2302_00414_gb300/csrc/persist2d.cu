@@ -10,7 +10,7 @@
 // queue is a list of segments (a run of spread units, or one job's x or y blocks) in the kernel
 // parameters.
 //
-// Measured on the batched d = 2 workload (64 sets): 0.425 ms per step against 0.314 ms for the
+// Measured on the batched d = 2 workload (64 sets): 0.416 ms per step against 0.311 ms for the
 // staged kernels in graph branches.  The spread units run at twelve warps per SM (three CTAs of the registers that
 // both kinds of unit need), where the staged spread runs at twenty, the FFT blocks as four-warp CTAs at that
 // occupancy, where the staged passes run eight-warp blocks at four or five per SM, and the overlap does not
