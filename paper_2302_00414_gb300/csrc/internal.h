@@ -149,27 +149,28 @@ bool fault(unsigned bit);
 
 // Allow launches of kernel K with `bytes` of dynamic shared memory.  A kernel's limit is one per process and device, not
 // per launch: set to each launch's own size, one host thread lowered it between another's setting and launch, which then
-// failed.  It goes up once, to all that a block can have beside the kernel's static arrays, and stays; the launch's
-// own size alone decides what it takes and how many blocks an SM holds.
+// failed.  Every call sets it to the same value, all that a block can have beside the kernel's static arrays (the
+// launch's own size alone decides what it takes and how many blocks an SM holds); set each time, it outlives a device
+// reset.  Only that value is remembered, which no reset changes.
 template <auto K>
 infft_status smem_limit(size_t bytes) {
-    static std::atomic<int> limit[64];   // by device; 0: not raised yet (threads that meet here set the same value)
+    static std::atomic<int> most[64];   // by device; 0: not looked up yet
     int dev = 0;
     INFFT_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) { set_error("device %d out of range", dev); return INFFT_EINVAL; }
-    int have = limit[dev].load(std::memory_order_acquire);
+    int have = most[dev].load(std::memory_order_relaxed);
     if (have == 0) {
         cudaFuncAttributes a;
         INFFT_CUDA(cudaFuncGetAttributes(&a, K));
         INFFT_CUDA(cudaDeviceGetAttribute(&have, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         have -= (int)a.sharedSizeBytes;
-        INFFT_CUDA(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, have));
-        limit[dev].store(have, std::memory_order_release);
+        most[dev].store(have, std::memory_order_relaxed);
     }
     if (bytes > (size_t)have) {
         set_error("a block needs %zu bytes of shared memory, the device gives %d", bytes, have);
         return INFFT_ECUDA;
     }
+    INFFT_CUDA(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, have));
     return INFFT_OK;
 }
 
